@@ -502,6 +502,7 @@ lbm_status lbm_nphase_create(const lbm_nphase_params *p, void *ws,
   g.err = (int *)(base + L.err);
   g.grad_scheme = p->grad_scheme;
   g.use_tma = false;
+  g.step64 = tma_allowed() && h->prec == LBM_FP64 && p->lattice == 0;
   g.march3 = tma_allowed() && !h->nonunif && p->lattice == 1;
   g.tma3 = g.march3 && h->prec == LBM_FP32 &&
            lbm::encode_tma3_f32(k, g, tensor_map_encoder());

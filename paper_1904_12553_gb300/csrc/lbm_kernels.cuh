@@ -1626,12 +1626,20 @@ __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
   }
 }
 
+}  // namespace lbm
+
+#include "lbm_step64.cuh"
+
+namespace lbm {
+
 // ---------------------------------------------------------------------------
 // Host-side launchers for one precision.
 // ---------------------------------------------------------------------------
 template <int P, int NP, bool NU, bool WALL>
 cudaError_t launch_tile_t(const Consts &c, const Grid &g, int cur, int mode,
                           const Outputs &o, cudaStream_t s) {
+  if constexpr (P == LBM_FP64)
+    if (mode == MODE_STEP && g.step64) return launch_step64<NP, NU, WALL>(c, g, cur, s);
   const KArgs<P> a = make_args<P>(c, g, cur, mode, o);
   if constexpr (P != LBM_FP64 && !NU) {
     if (mode == MODE_STEP && g.use_tma && g.grad_scheme == 0) {
