@@ -139,9 +139,11 @@ lbm_status lbm_nphase_init(lbm_nphase_t *h, const double *c, const double *u,
 /* Advance nsteps >= 0 time steps (asynchronous on the handle's stream). Each
  * step is one fused kernel: zeroth moments (Eq. N28), chemical potentials
  * (Eqs. N17, N18, N31), forces, u and p (Eqs. N22_1, N23), both
- * collisions (Eqs. 24, N24) and streaming. From nsteps >= 4 on, pairs of
- * steps are replayed from a CUDA graph captured on the handle's first such
- * call (on a private stream; call it outside any capture of your own).
+ * collisions (Eqs. 24, N24) and streaming (two for FP64 grids with unequal
+ * densities or Eq. N40). From nsteps >= 4 on, pairs of steps are replayed
+ * from a CUDA graph captured on the handle's first such call (on a private
+ * stream; call it outside any capture of your own), from nsteps >= 32 on
+ * also chains of 32.
  * Errors: LBM_ESTATE before init or after LBM_EUNSTABLE, LBM_ECUDA. */
 lbm_status lbm_nphase_step(lbm_nphase_t *h, int64_t nsteps);
 

@@ -566,30 +566,51 @@ static cudaError_t step_once(lbm_nphase_t *h, cudaStream_t s, int cur) {
                           h->nonunif, h->wall, s);
 }
 
-// Two steps (buffer p -> p^1 -> p) captured as a graph, for p = 0 and 1.
-static cudaError_t build_step_graphs(lbm_nphase_t *h) {
+// Steps per graph: a pair, and a chain for long runs. Back to back, graphs
+// start at multiples of about 2 us on GB300, kernels inside one graph follow
+// each other at once (0.55 us for empty ones), so a chain saves a small
+// grid's step up to 1 us: FP32 256^2 with walls 6.16 us per step in pairs,
+// 5.39 in chains of 8, 5.26 of 16, 5.27 of 32, 5.24 of 64. Chains of 32 are
+// captured when a call of at least that many steps first asks for one.
+constexpr int kChain[2] = {2, 32};
+
+// kChain[l] steps from buffer p (an even number: back to p) as a graph.
+static cudaError_t build_step_graph(lbm_nphase_t *h, int l, int p) {
   cudaError_t e = cudaSuccess;
   if (!h->cap) e = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking);
-  for (int p = 0; p < 2 && e == cudaSuccess; ++p) {
-    cudaGraph_t graph = nullptr;
-    e = cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) break;
-    cudaError_t e1 = step_once(h, h->cap, p);
-    cudaError_t e2 = step_once(h, h->cap, p ^ 1);
-    e = cudaStreamEndCapture(h->cap, &graph);
-    if (e == cudaSuccess && e1 != cudaSuccess) e = e1;
-    if (e == cudaSuccess && e2 != cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&h->gexec[p], graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-  }
+  if (e == cudaSuccess) e = cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return e;
+  cudaGraph_t graph = nullptr;
+  cudaError_t es = cudaSuccess;
+  for (int t = 0; t < kChain[l] && es == cudaSuccess; ++t) es = step_once(h, h->cap, p ^ (t & 1));
+  e = cudaStreamEndCapture(h->cap, &graph);
+  if (e == cudaSuccess) e = es;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&h->gexec[l][p], graph, 0);
+  if (graph) cudaGraphDestroy(graph);
   return e;
+}
+
+// Whether a chain from the current buffer is there, built now if need be. Not
+// while the caller captures the handle's stream: such calls replay pairs.
+static bool have_chain(lbm_nphase_t *h) {
+  if (h->gexec[1][h->cur]) return true;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (h->no_chain || cudaStreamIsCapturing(h->stream, &st) != cudaSuccess ||
+      st != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  if (build_step_graph(h, 1, h->cur) == cudaSuccess) return true;
+  cudaGetLastError();
+  h->no_chain = true;
+  return false;
 }
 
 lbm_status lbm_nphase_step(lbm_nphase_t *h, int64_t nsteps) {
   if (!h || nsteps < 0) return LBM_EINVAL;
   if (!h->initialized || h->unstable) return LBM_ESTATE;
   int64_t t = 0;
-  if (nsteps >= 4 && !h->gexec[0]) {
+  if (nsteps >= 4 && !h->gexec[0][0]) {
     // one step launched directly first: the launchers' one-time setup
     // (shared-memory attributes, occupancy) then runs outside the capture
     cudaError_t e = step_once(h, h->stream, h->cur);
@@ -597,15 +618,16 @@ lbm_status lbm_nphase_step(lbm_nphase_t *h, int64_t nsteps) {
     h->cur ^= 1;
     ++h->steps;
     ++t;
-    e = build_step_graphs(h);
+    for (int p = 0; p < 2 && e == cudaSuccess; ++p) e = build_step_graph(h, 0, p);
     if (e != cudaSuccess) return cuda_fail(h, e);
   }
-  if (h->gexec[0])
-    for (; t + 2 <= nsteps; t += 2) {
-      cudaError_t e = cudaGraphLaunch(h->gexec[h->cur], h->stream);
-      if (e != cudaSuccess) return cuda_fail(h, e);
-      h->steps += 2;
-    }
+  if (h->gexec[0][0])
+    for (int l = 1; l >= 0; --l)
+      for (; t + kChain[l] <= nsteps && (l == 0 || have_chain(h)); t += kChain[l]) {
+        cudaError_t e = cudaGraphLaunch(h->gexec[l][h->cur], h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e);
+        h->steps += kChain[l];
+      }
   for (; t < nsteps; ++t) {
     cudaError_t e = step_once(h, h->stream, h->cur);
     if (e != cudaSuccess) return cuda_fail(h, e);
@@ -816,8 +838,9 @@ int lbm_nphase_cuda_error(const lbm_nphase_t *h) { return h ? h->cuda_err : 0; }
 
 lbm_status lbm_nphase_destroy(lbm_nphase_t *h) {
   if (!h) return LBM_OK;
-  for (int p = 0; p < 2; ++p)
-    if (h->gexec[p]) cudaGraphExecDestroy(h->gexec[p]);
+  for (int l = 0; l < 2; ++l)
+    for (int p = 0; p < 2; ++p)
+      if (h->gexec[l][p]) cudaGraphExecDestroy(h->gexec[l][p]);
   if (h->cap) cudaStreamDestroy(h->cap);
   delete h;
   return LBM_OK;

@@ -143,7 +143,8 @@ struct lbm_nphase_t {
   int64_t steps;
   int cuda_err;
   cudaStream_t cap;            // private stream for graph capture
-  cudaGraphExec_t gexec[2];    // two steps starting at buffer 0 / 1
+  cudaGraphExec_t gexec[2][2]; // a pair, a chain of steps from buffer 0 / 1
+  bool no_chain;               // the chain's capture failed: pairs only
 };
 
 namespace lbm {
