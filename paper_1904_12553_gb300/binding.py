@@ -374,6 +374,8 @@ class Solver:
 
     @property
     def step_kernel(self) -> str:
+        """Name of the step's kernels (2 and 3: the D3Q15 kernels, split or,
+        for large FP32 boxes, z-marching)."""
         return {1: "pipelined (TMA)", 2: "z-marching 3-D",
                 3: "z-marching 3-D (TMA)"}.get(
             lbm_nphase_uses_pipelined_kernel(self.handle), "generic tile")

@@ -38,11 +38,23 @@ static_assert(c3x(opp3(8)) == -c3x(8) && c3y(opp3(8)) == -c3y(8) &&
                   c3y(opp3(13)) == -c3y(13) && c3z(opp3(9)) == -c3z(9),
               "D3Q15 opposites");
 
+// The 7 pairs of opposite directions: pair of k, and a pair's first direction
+// (faces 1-3, corners 7-10).
+__host__ __device__ constexpr int mag3_k(int j) { return j < 3 ? j + 1 : j + 4; }
+__host__ __device__ constexpr int mag3(int k) {
+  return (k < opp3(k) ? k : opp3(k)) <= 3 ? (k < opp3(k) ? k : opp3(k)) - 1
+                                          : (k < opp3(k) ? k : opp3(k)) - 4;
+}
+static_assert(opp3(7) == 11 && opp3(8) == 12 && opp3(9) == 13 && opp3(10) == 14,
+              "corner pairs");
+
 constexpr int BX3 = 32, BY3 = 4, BZ3 = 2, NT3 = BX3 * BY3 * BZ3;
+constexpr int MX3 = 32, MY3 = 8, MT3 = MX3 * MY3;
 
 template <int P> struct KArgs3 {
   KArgs<P> a;  // pointers, constants (u_in, u_out hold 3 planes)
   int nz;
+  typename Prec<P>::T *C;  // C_i of the split step with unequal densities
 };
 
 // Stencils of Eq. N31 on a shared box (strides W, W * H): D3Q15 sums folded
@@ -154,59 +166,121 @@ template <bool WALL> struct Nb3 {
     lo = WALL && y == 0;
     hi = WALL && y == ny - 1;
   }
+  template <typename S> __device__ __forceinline__ const S *src(const S *plane, int k) const {
+    return plane + src(k);
+  }
   __device__ __forceinline__ size_t src(int k) const {
     const int cx = c3x(k), cy = c3y(k), cz = c3z(k);
     if (WALL && ((cy > 0 && lo) || (cy < 0 && hi))) return q;
     return pz[1 - cz] + ry[1 - cy] + (size_t)xv[1 - cx];
   }
+  // where population k goes: the node of slot dk(k) in a plane array
+  __device__ __forceinline__ int dk(int k) const {
+    return WALL && ((c3y(k) < 0 && lo) || (c3y(k) > 0 && hi)) ? opp3(k) : k;
+  }
+  template <typename S> __device__ __forceinline__ S *dst(S *plane, int k) const {
+    if (WALL && ((c3y(k) < 0 && lo) || (c3y(k) > 0 && hi))) return plane + q;
+    return plane + (pz[1 + c3z(k)] + ry[1 + c3y(k)] + (size_t)xv[1 + c3x(k)]);
+  }
+  template <typename S> __device__ __forceinline__ S *own(S *plane) const { return plane + q; }
+  // neighbour (x, y, z) + c_k of a stencil (a wall's ghost row repeats its row)
+  template <typename S> __device__ __forceinline__ const S *nb(const S *plane, int k) const {
+    return plane + (pz[1 + c3z(k)] + ry[1 + c3y(k)] + (size_t)xv[1 + c3x(k)]);
+  }
+};
+// The same for a node away from the walls, split into the z planes' offsets
+// (one value for the whole CTA) and 32-bit offsets of the 3 x 3 neighbours
+// within a plane, computed once for all planes a thread walks: an access then
+// takes its address from a uniform base and one register. Planes of less than
+// 2^32 bytes (the launcher checks).
+struct Off3 {
+  size_t pz[3];
+  unsigned e[3][3];  // [dy + 1][dx + 1], in nodes
+  __device__ __forceinline__ void set_xy(int x, int y, int nx, int ny) {
+    const int xv[3] = {x == 0 ? nx - 1 : x - 1, x, x + 1 >= nx ? x + 1 - nx : x + 1};
+    const int yv[3] = {y == 0 ? ny - 1 : y - 1, y, y + 1 >= ny ? y + 1 - ny : y + 1};
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) e[j][i] = (unsigned)yv[j] * (unsigned)nx + (unsigned)xv[i];
+  }
+  __device__ __forceinline__ void set_z(int z, int nz, size_t plane) {
+    pz[0] = (size_t)(z == 0 ? nz - 1 : z - 1) * plane;
+    pz[1] = (size_t)z * plane;
+    pz[2] = (size_t)(z + 1 >= nz ? z + 1 - nz : z + 1) * plane;
+  }
+  template <typename S> static __device__ __forceinline__ S *at(S *base, unsigned node) {
+    return (S *)((char *)base + (size_t)(node * (unsigned)sizeof(S)));
+  }
+  // slot k's source, population k's destination, the node itself
+  template <typename S> __device__ __forceinline__ const S *src(const S *plane, int k) const {
+    return at(plane + pz[1 - c3z(k)], e[1 - c3y(k)][1 - c3x(k)]);
+  }
+  template <typename S> __device__ __forceinline__ S *dst(S *plane, int k) const {
+    return at(plane + pz[1 + c3z(k)], e[1 + c3y(k)][1 + c3x(k)]);
+  }
+  template <typename S> __device__ __forceinline__ S *own(S *plane) const {
+    return at(plane + pz[1], e[1][1]);
+  }
+  template <typename S> __device__ __forceinline__ const S *nb(const S *plane, int k) const {
+    return at(plane + pz[1 + c3z(k)], e[1 + c3y(k)][1 + c3x(k)]);
+  }
+  static __device__ __forceinline__ int dk(int k) { return k; }
 };
 
-// phi_i of every phase at node (x, y, z) = q from the stored values (FP64:
-// sum of the 15; other forms: phi(t-1) + (d_0 + sum_k h_k), TwoSum error
-// dropped). 16-bit forms decode slot k with u(t-1), phi(t-1) of its source,
-// looked up once for all phases. With OWN, the node's decoded h^i_1..14 and
-// g_1..14 also go to own[slot * stride] (slot i * 14 + k - 1, then
-// (NP - 1) * 14 + 13 + k for g), for the node's own step to read back.
-template <int P, int NP, bool WALL, bool OWN = false>
-__device__ __forceinline__ void node_phis3(const KArgs<P> &a, int nz, int x,
-                                           int y, int z, size_t q,
-                                           typename Prec<P>::T (&phi)[NP],
-                                           typename Prec<P>::T *own = nullptr,
-                                           int stride = 0) {
+// Destinations of one node's populations as indices, for tile3_kernel.
+template <bool WALL> struct Dst3 {
+  size_t q, d[15];
+  int kk[15];
+  __device__ __forceinline__ Dst3(int x, int y, int z, size_t q_, int nx, int ny, int nz) {
+    q = q_;
+#pragma unroll
+    for (int k = 1; k < 15; ++k) {
+      const int yy = y + c3y(k);
+      if (WALL && (yy < 0 || yy >= ny)) {
+        d[k] = q;
+        kk[k] = opp3(k);
+      } else {
+        d[k] = ((size_t)wrap(z + c3z(k), nz) * ny + wrap_y<WALL>(yy, ny)) * nx +
+               wrap(x + c3x(k), nx);
+        kk[k] = k;
+      }
+    }
+  }
+  __device__ __forceinline__ int dk(int k) const { return kk[k]; }
+  template <typename S> __device__ __forceinline__ S *dst(S *plane, int k) const {
+    return plane + d[k];
+  }
+  template <typename S> __device__ __forceinline__ S *own(S *plane) const { return plane + q; }
+};
+
+// phi_i of every phase at a node from the stored values (FP64: sum of the 15;
+// other forms: phi(t-1) + (d_0 + sum_k h_k), TwoSum error dropped). 16-bit
+// forms decode slot k with u(t-1), phi(t-1) of its source, looked up once for
+// all phases.
+template <int P, int NP, typename At>
+__device__ __forceinline__ void node_phis3_at(const KArgs<P> &a, const At &at,
+                                              typename Prec<P>::T (&phi)[NP]) {
   typedef typename Prec<P>::T T;
   const size_t V = a.V;
   T small[NP];
 #pragma unroll
-  for (int i = 0; i < NP; ++i) small[i] = ldg(a.h0_in + (size_t)i * V + q);
-  const Nb3<WALL> nb(x, y, z, q, a.nx, a.ny, nz);
+  for (int i = 0; i < NP; ++i) small[i] = ldg(at.own(a.h0_in + (size_t)i * V));
 #pragma unroll
   for (int k = 1; k < 15; ++k) {
-    T cu = T(0), ux = T(0), uy = T(0), uz = T(0);
-    size_t qs = q;
-    if constexpr (Prec<P>::REF) {
-      qs = nb.src(k);
-      ux = ldg(a.u_in + qs);
-      uy = ldg(a.u_in + V + qs);
-      uz = ldg(a.u_in + 2 * V + qs);
-      cu = cdotu3(k, ux, uy, uz);
-    }
+    T cu = T(0);
+    if constexpr (Prec<P>::REF)
+      cu = cdotu3(k, ldg(at.src(a.u_in, k)), ldg(at.src(a.u_in + V, k)),
+                  ldg(at.src(a.u_in + 2 * V, k)));
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      T x_ = load_hm3<P>(a, i, k, q);
+      T x_ = to_T(ldg(at.own(a.hm_in + (size_t)(i * 14 + k - 1) * V)));
       if constexpr (Prec<P>::REF)
-        x_ = __fadd_rn(x_, adv_units(cu, ldg(a.pp_in + (size_t)i * V + qs), T(3) * a.sh_st));
-      if constexpr (OWN) own[(i * 14 + k - 1) * stride] = x_;
+        x_ = __fadd_rn(x_, adv_units(cu, ldg(at.src(a.pp_in + (size_t)i * V, k)), T(3) * a.sh_st));
       if constexpr (Prec<P>::MIX)
         small[i] = __fmaf_rn(w3_of<T>(k) * a.sh_ld, x_, small[i]);
       else
         small[i] = __fadd_rn_T(small[i], x_);
-    }
-    if constexpr (OWN) {
-      T gk = to_T(ldg(a.gm_in + (size_t)(k - 1) * V + q));
-      if constexpr (Prec<P>::REF)
-        gk = __fadd_rn(gk, g_ref3p(cu, ux, uy, uz, ldg(a.u_in + 3 * V + qs),
-                                   a.rho_base * a.sg_st, T(3) * a.sg_st));
-      own[(NP * 14 + k - 1) * stride] = gk;
     }
   }
 #pragma unroll
@@ -214,8 +288,14 @@ __device__ __forceinline__ void node_phis3(const KArgs<P> &a, int nz, int x,
     if constexpr (P == LBM_FP64)
       phi[i] = small[i];
     else
-      phi[i] = __fadd_rn(ldg(a.pp_in + (size_t)i * V + q), small[i]);
+      phi[i] = __fadd_rn(ldg(at.own(a.pp_in + (size_t)i * V)), small[i]);
   }
+}
+template <int P, int NP, bool WALL>
+__device__ __forceinline__ void node_phis3(const KArgs<P> &a, int nz, int x,
+                                           int y, int z, size_t q,
+                                           typename Prec<P>::T (&phi)[NP]) {
+  node_phis3_at<P, NP>(a, Nb3<WALL>(x, y, z, q, a.nx, a.ny, nz), phi);
 }
 
 template <bool WALL>
@@ -232,58 +312,36 @@ template <int P, int NP> struct Own3 {
   T h[NP][15], g[15], pp[NP], up[3];
 };
 
-template <int P, int NP, bool WALL>
-__device__ __forceinline__ void load_own3(const KArgs<P> &a, int nz, int x,
-                                          int y, int z, size_t q,
-                                          Own3<P, NP> &o) {
+template <int P, int NP, typename At>
+__device__ __forceinline__ void load_own3(const KArgs<P> &a, const At &at, Own3<P, NP> &o) {
   typedef typename Prec<P>::T T;
   const size_t V = a.V;
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
-    o.h[i][0] = ldg(a.h0_in + (size_t)i * V + q);
+    o.h[i][0] = ldg(at.own(a.h0_in + (size_t)i * V));
 #pragma unroll
-    for (int k = 1; k < 15; ++k) o.h[i][k] = load_hm3<P>(a, i, k, q);
-    o.pp[i] = ldg(a.pp_in + (size_t)i * V + q);
+    for (int k = 1; k < 15; ++k)
+      o.h[i][k] = to_T(ldg(at.own(a.hm_in + (size_t)(i * 14 + k - 1) * V)));
+    o.pp[i] = ldg(at.own(a.pp_in + (size_t)i * V));
   }
 #pragma unroll
-  for (int k = 1; k < 15; ++k) o.g[k] = to_T(ldg(a.gm_in + (size_t)(k - 1) * V + q));
+  for (int k = 1; k < 15; ++k) o.g[k] = to_T(ldg(at.own(a.gm_in + (size_t)(k - 1) * V)));
   if constexpr (Prec<P>::REF) {
-    const Nb3<WALL> nb(x, y, z, q, a.nx, a.ny, nz);
 #pragma unroll
     for (int k = 1; k < 15; ++k) {
-      const size_t qs = nb.src(k);
-      const T ux = ldg(a.u_in + qs), uy = ldg(a.u_in + V + qs),
-              uz = ldg(a.u_in + 2 * V + qs);
+      const T ux = ldg(at.src(a.u_in, k)), uy = ldg(at.src(a.u_in + V, k)),
+              uz = ldg(at.src(a.u_in + 2 * V, k));
       const T cu = cdotu3(k, ux, uy, uz);
 #pragma unroll
       for (int i = 0; i < NP; ++i)
-        o.h[i][k] = __fadd_rn(o.h[i][k], adv_units(cu, ldg(a.pp_in + (size_t)i * V + qs),
+        o.h[i][k] = __fadd_rn(o.h[i][k], adv_units(cu, ldg(at.src(a.pp_in + (size_t)i * V, k)),
                                                    T(3) * a.sh_st));
-      o.g[k] = __fadd_rn(o.g[k], g_ref3p(cu, ux, uy, uz, ldg(a.u_in + 3 * V + qs),
+      o.g[k] = __fadd_rn(o.g[k], g_ref3p(cu, ux, uy, uz, ldg(at.src(a.u_in + 3 * V, k)),
                                          a.rho_base * a.sg_st, T(3) * a.sg_st));
     }
   }
 #pragma unroll
-  for (int d = 0; d < 3; ++d) o.up[d] = a.u_in[(size_t)d * V + q];
-}
-
-// The same values, h and g decoded by node_phis3<..., OWN> into own[].
-template <int P, int NP>
-__device__ __forceinline__ void load_own3c(const KArgs<P> &a, size_t q,
-                                           const typename Prec<P>::T *own,
-                                           int stride, Own3<P, NP> &o) {
-  const size_t V = a.V;
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    o.h[i][0] = ldg(a.h0_in + (size_t)i * V + q);
-#pragma unroll
-    for (int k = 1; k < 15; ++k) o.h[i][k] = own[(i * 14 + k - 1) * stride];
-    o.pp[i] = ldg(a.pp_in + (size_t)i * V + q);
-  }
-#pragma unroll
-  for (int k = 1; k < 15; ++k) o.g[k] = own[(NP * 14 + k - 1) * stride];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) o.up[d] = a.u_in[(size_t)d * V + q];
+  for (int d = 0; d < 3; ++d) o.up[d] = ldg(at.own(a.u_in + (size_t)d * V));
 }
 
 // phi_i from a node's values in registers, summed in the order of node_phis3.
@@ -351,30 +409,20 @@ __device__ __forceinline__ void macros3(
 // Collisions of one D3Q15 node (Eqs. 24, N24 with Eqs. 25, N20_1, N25-N27),
 // folded as in the D2Q9 kernels, and push streaming; phi(t) and u(t) become
 // the next step's phi(t-1) and u(t-1).
-template <int P, int NP, bool NU, bool WALL>
+template <int P, int NP, bool NU, typename At>
 __device__ __forceinline__ void collide3(
-    const KArgs<P> &a, int nz, const typename Prec<P>::T *ph,
+    const KArgs<P> &a, const At &at, const typename Prec<P>::T *ph,
     const typename Prec<P>::T *Cv, typename Prec<P>::T rho,
     const typename Prec<P>::T *gr, const typename Prec<P>::T *J,
     const Own3<P, NP> &o, const typename Prec<P>::T (&u)[3],
     const typename Prec<P>::T (&F)[3], typename Prec<P>::T uu,
-    typename Prec<P>::T pr, size_t q, int gx, int gy, int gz) {
+    typename Prec<P>::T pr, bool store_phi = true) {
   typedef typename Prec<P>::T T;
-  const int nx = a.nx, ny = a.ny;
   const size_t V = a.V;
-  size_t dst[15];
+  // population k goes to slot dk[k] of the node at.dst points to
   int dk[15];
 #pragma unroll
-  for (int k = 1; k < 15; ++k) {
-    const int yy = gy + c3y(k);
-    if (WALL && (yy < 0 || yy >= ny)) {
-      dst[k] = q;
-      dk[k] = opp3(k);
-    } else {
-      dst[k] = node3<WALL>(gx + c3x(k), yy, gz + c3z(k), nx, ny, nz);
-      dk[k] = k;
-    }
-  }
+  for (int k = 1; k < 15; ++k) dk[k] = at.dk(k);
   constexpr bool MIX = Prec<P>::MIX;
   const T tg = a.tg_inv, ff = a.ffac;
   const T uF = u[0] * F[0] + u[1] * F[1] + u[2] * F[2];
@@ -383,6 +431,22 @@ __device__ __forceinline__ void collide3(
   const T B1 = T(3) * tg * rho, B2 = T(4.5) * tg * rho;
   const T C1 = T(3) * ff, D1 = T(9) * ff, E1 = T(3) * ff, E2 = T(4.5) * ff * a.jfac;
   const T keep_g = T(1) - tg;
+  // 16-bit forms: the writer's references, formed once per magnitude of c_k.u
+  // (as cdotu3 rounds it, it is +-um[j]; the rounded products 3 c.u, (c.u)^2
+  // and (c.u) phi are odd or even in it), the bits of g_ref3p / adv_units
+  T um[7], g3u[7], g45[7], gv[15];
+  T uut = T(0), p3 = T(0);
+  if constexpr (MIX) {
+    uut = __fmul_rn(T(-1.5), __fadd_rn(__fadd_rn(__fmul_rn(u[0], u[0]), __fmul_rn(u[1], u[1])),
+                                       __fmul_rn(u[2], u[2])));
+    p3 = __fmul_rn(pr, T(3) * a.sg_st);
+#pragma unroll
+    for (int j = 0; j < 7; ++j) {
+      um[j] = cdotu3(mag3_k(j), u[0], u[1], u[2]);
+      g3u[j] = __fmul_rn(T(3), um[j]);
+      g45[j] = __fmul_rn(T(4.5), __fmul_rn(um[j], um[j]));
+    }
+  }
 #pragma unroll
   for (int k = 1; k < 15; ++k) {
     const T cx = T(c3x(k)), cy = T(c3y(k)), cz = T(c3z(k));
@@ -393,14 +457,23 @@ __device__ __forceinline__ void collide3(
       inner += E1 * (cx * gr[0] + cy * gr[1] + cz * gr[2]) +
                E2 * (cx * J[0] + cy * J[1] + cz * J[2]);
     const T t = A0 + C1 * cF + cu * inner;
-    if constexpr (MIX)
-      a.gm_out[(size_t)(dk[k] - 1) * V + dst[k]] = to_S<typename Prec<P>::Sm>(
-          keep_g * o.g[k] + a.sg_st * t -
-          (Prec<P>::REF ? g_ref3p(cdotu3(dk[k], u[0], u[1], u[2]), u[0], u[1], u[2], pr,
-                                  a.rho_base * a.sg_st, T(3) * a.sg_st)
-                        : T(0)));
-    else
-      a.gm_out[(size_t)(dk[k] - 1) * V + dst[k]] = keep_g * o.g[k] + w3_of<T>(k) * t;
+    if constexpr (MIX) {
+      const int j = mag3(k);
+      const bool neg = (mag3_k(j) != k) != (dk[k] != k);  // sign of c_dk.u against um
+      const T sr = __fadd_rn(neg ? -g3u[j] : g3u[j], g45[j]);
+      const T ref = __fadd_rn(__fmul_rn(__fadd_rn(sr, uut), a.rho_base * a.sg_st), p3);
+      gv[k] = keep_g * o.g[k] + a.sg_st * t - ref;
+    } else
+      *at.dst(a.gm_out + (size_t)(dk[k] - 1) * V, k) = keep_g * o.g[k] + w3_of<T>(k) * t;
+  }
+  if constexpr (MIX) {  // converted two at a time
+#pragma unroll
+    for (int k = 1; k < 15; k += 2) {
+      typename Prec<P>::Sm s0, s1;
+      to_S2(gv[k], gv[k + 1], s0, s1);
+      *at.dst(a.gm_out + (size_t)(dk[k] - 1) * V, k) = s0;
+      *at.dst(a.gm_out + (size_t)(dk[k + 1] - 1) * V, k + 1) = s1;
+    }
   }
   const T *up = o.up;
 #pragma unroll
@@ -419,23 +492,34 @@ __device__ __forceinline__ void collide3(
     T moving_sum = T(0), perr;
     // phi's rounding error of this node, from its values as loaded
     node_phi3r<P>(o.h[i], pp, perr, a.sh_ld);
+    if constexpr (MIX) {
+      // relative to the advective part at this node, the slot's source;
+      // converted two at a time, the mass balance with each value as the
+      // reader will decode it
+      T um3[7], hv[15], rf[15];
+      typename Prec<P>::Sm sv[15];
 #pragma unroll
-    for (int k = 1; k < 15; ++k) {
-      const T t = al + T(c3x(k)) * b[0] + T(c3y(k)) * b[1] + T(c3z(k)) * b[2];
-      const T hk = o.h[i][k];
-      const size_t oo = ((size_t)(i * 14 + dk[k] - 1)) * V + dst[k];
-      if constexpr (MIX) {
-        // relative to the advective part at this node, the slot's source
-        const T ref = Prec<P>::REF
-                          ? adv_units(cdotu3(dk[k], u[0], u[1], u[2]), ph[i], T(3) * a.sh_st)
-                          : T(0);
-        const auto sv = to_S<typename Prec<P>::Sm>(keep * hk + t - ref);
-        a.hm_out[oo] = sv;
-        moving_sum = __fmaf_rn(w3_of<T>(k) * a.sh_ld, __fadd_rn(to_T(sv), ref),
-                               moving_sum);
-      } else {
-        const T hs = keep * hk + w3_of<T>(k) * t;
-        a.hm_out[oo] = hs;
+      for (int j = 0; j < 7; ++j) um3[j] = adv_units(um[j], ph[i], T(3) * a.sh_st);
+#pragma unroll
+      for (int k = 1; k < 15; ++k) {
+        const T t = al + T(c3x(k)) * b[0] + T(c3y(k)) * b[1] + T(c3z(k)) * b[2];
+        const int j = mag3(k);
+        rf[k] = (mag3_k(j) != k) != (dk[k] != k) ? -um3[j] : um3[j];
+        hv[k] = keep * o.h[i][k] + t - rf[k];
+      }
+#pragma unroll
+      for (int k = 1; k < 15; k += 2) to_S2(hv[k], hv[k + 1], sv[k], sv[k + 1]);
+#pragma unroll
+      for (int k = 1; k < 15; ++k) {
+        *at.dst(a.hm_out + (size_t)(i * 14 + dk[k] - 1) * V, k) = sv[k];
+        moving_sum = __fmaf_rn(w3_of<T>(k) * a.sh_ld, __fadd_rn(to_T(sv[k]), rf[k]), moving_sum);
+      }
+    } else {
+#pragma unroll
+      for (int k = 1; k < 15; ++k) {
+        const T t = al + T(c3x(k)) * b[0] + T(c3y(k)) * b[1] + T(c3z(k)) * b[2];
+        const T hs = keep * o.h[i][k] + w3_of<T>(k) * t;
+        *at.dst(a.hm_out + (size_t)(i * 14 + dk[k] - 1) * V, k) = hs;
         moving_sum = __fadd_rn_T(moving_sum, hs);
       }
     }
@@ -445,12 +529,12 @@ __device__ __forceinline__ void collide3(
     } else {
       rest = __fsub_rn(perr, moving_sum);
     }
-    a.h0_out[(size_t)i * V + q] = rest;
-    a.pp_out[(size_t)i * V + q] = ph[i];
+    *at.own(a.h0_out + (size_t)i * V) = rest;
+    if (store_phi) *at.own(a.pp_out + (size_t)i * V) = ph[i];
   }
 #pragma unroll
-  for (int d = 0; d < 3; ++d) a.u_out[(size_t)d * V + q] = u[d];
-  if constexpr (Prec<P>::REF) a.u_out[3 * V + q] = pr;
+  for (int d = 0; d < 3; ++d) *at.own(a.u_out + (size_t)d * V) = u[d];
+  if constexpr (Prec<P>::REF) *at.own(a.u_out + 3 * V) = pr;
 }
 
 template <int P, int NP, bool NU, bool WALL>
@@ -563,8 +647,8 @@ __global__ void __launch_bounds__(NT3, P == LBM_FP64 ? 1 : 2)
   }
   // own-node values (node 0 stands in for inactive threads)
   Own3<P, NP> own;
-  load_own3<P, NP, WALL>(a, nz, active ? gx : 0, active ? gy : 0, active ? gz : 0,
-                         q, own);
+  load_own3<P, NP>(
+      a, Nb3<WALL>(active ? gx : 0, active ? gy : 0, active ? gz : 0, q, nx, ny, nz), own);
   T F[3], u[3], uu, pr;
   macros3<P, NP>(a, gp, Cv, rho, gr, own.g, u, F, uu, pr);
   if (a.mode == MODE_MOMENTS) {
@@ -602,29 +686,144 @@ __global__ void __launch_bounds__(NT3, P == LBM_FP64 ? 1 : 2)
   }
   if (!active) return;
 
-  collide3<P, NP, NU, WALL>(a, nz, ph, Cv, rho, gr, J, own, u, F, uu, pr, q,
-                            gx, gy, gz);
+  collide3<P, NP, NU>(a, Dst3<WALL>(gx, gy, gz, q, nx, ny, nz), ph, Cv, rho, gr, J, own, u, F,
+                      uu, pr);
 }
 
 // ---------------------------------------------------------------------------
-// z-marching step kernel (equal densities, central scheme). A CTA owns a
-// 32 x 8 column of the grid and walks a slab of z planes. phi of plane z + 1
-// is summed on the column's tile and its xy ring into a rolling window of
-// three planes (z - 1, z, z + 1) in shared memory, so a node's phi is summed
-// once per slab (plus the 84 ring positions per 256 nodes of a plane)
-// instead of on a 3-D halo box around every tile; the 14 stencil neighbours
-// of a node of plane z then come from the window. The per-node step is the
-// one of tile3_kernel (macros3, collide3).
+// The step split in two kernels (three with unequal densities): phi(t) of
+// every node to the next step's phi(t-1) array (phi3_kernel), C_i from its
+// stencils (pot3_kernel, unequal densities), then the step of every node from
+// the stencils of both in memory (step3_kernel). No barriers, and nothing is
+// computed twice: a tile with its halo sums phi on 3.2 positions per node (6.8
+// with unequal densities), a column marched in z on 1.33 and two more planes
+// per slab, and in the 16-bit forms, which are bound by instruction issue, a
+// position costs the decode of 14 slots from their sources. It costs one more
+// read of h; the stencils' reads are L1 and L2 hits.
+// us per step before (a z-marching kernel with the column's decoded values in
+// shared memory, or the tile kernel) -> now: BF16 128^3 N = 3 with walls 409
+// -> 243 (63 + 180), 160^3 N = 4 829 -> 652; FP16 96^3 N = 5 334 -> 215; FP32
+// 128^3 N = 5 480 -> 365, 101 x 93 x 87 N = 3 118 -> 90, 33 x 29 x 31 27 ->
+// 7.9; FP64 64^3 N = 5 578 -> 476; FP32 96^3 N = 3, unequal densities 162 ->
+// 104. Blocks of one plane (32 x 8 x 1) gave the same, 104 -> 112 with
+// unequal densities.
 // ---------------------------------------------------------------------------
-constexpr int MX3 = 32, MY3 = 8, MT3 = MX3 * MY3;
-// dynamic shared memory of march3_kernel: 14 (N - 1) + 14 decoded values
-// per column, then the three-plane phi window (tile and xy ring)
-template <int P, int NP> __host__ __device__ constexpr size_t march3_cache_bytes() {
-  return (size_t)(NP * 14 + 14) * MT3 * sizeof(typename Prec<P>::T);
+
+// Eq. N31 on D3Q15 on a field in memory, pairs of opposite velocities summed
+// in the order of stencil3.
+template <typename T, typename At>
+__device__ __forceinline__ void stencil3m(const T *z, const At &at, T c, T *g, T &lap) {
+  T gx = T(0), gy = T(0), gz = T(0), l = T(0);
+#pragma unroll
+  for (int k = 1; k < 15; ++k) {
+    if (opp3(k) < k) continue;
+    const T p = *at.nb(z, k), m = *at.nb(z, opp3(k));
+    const T wd = w3_of<T>(k) * (p - m);
+    gx += T(c3x(k)) * wd;
+    gy += T(c3y(k)) * wd;
+    gz += T(c3z(k)) * wd;
+    l += w3_of<T>(k) * (p + m - T(2) * c);
+  }
+  g[0] = T(3) * gx;
+  g[1] = T(3) * gy;
+  g[2] = T(3) * gz;
+  lap = T(6) * l;
 }
-template <int P, int NP> __host__ __device__ constexpr size_t march3_smem() {
-  return march3_cache_bytes<P, NP>() +
-         (size_t)3 * NP * (MX3 + 2) * (MY3 + 2) * sizeof(typename Prec<P>::T);
+
+// Calls f(at) for the node of this thread, `at` an Off3 away from the walls.
+// Tiles of 32 x 4 x 2 nodes.
+template <bool WALL, typename F>
+__device__ __forceinline__ void for_node3(int nx, int ny, int nz, F f) {
+  const int x = blockIdx.x * BX3 + threadIdx.x, y = blockIdx.y * BY3 + threadIdx.y,
+            z = blockIdx.z * BZ3 + threadIdx.z;
+  if (x >= nx || y >= ny || z >= nz) return;
+  if (!WALL || (y > 0 && y < ny - 1)) {
+    Off3 o;
+    o.set_xy(x, y, nx, ny);
+    o.set_z(z, nz, (size_t)nx * ny);
+    f(o);
+  } else {
+    f(Nb3<WALL>(x, y, z, ((size_t)z * ny + y) * nx + x, nx, ny, nz));
+  }
+}
+
+template <int P, int NP, bool WALL>
+__global__ void __launch_bounds__(NT3) phi3_kernel(const KArgs3<P> A) {
+  typedef typename Prec<P>::T T;
+  const KArgs<P> &a = A.a;
+  for_node3<WALL>(a.nx, a.ny, A.nz, [&](const auto &at) {
+    T phv[NP];
+    node_phis3_at<P, NP>(a, at, phv);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) *at.own(a.pp_out + (size_t)i * a.V) = phv[i];
+  });
+}
+
+template <int P, int NP, bool WALL>
+__global__ void __launch_bounds__(NT3) pot3_kernel(const KArgs3<P> A) {
+  typedef typename Prec<P>::T T;
+  const KArgs<P> &a = A.a;
+  for_node3<WALL>(a.nx, a.ny, A.nz, [&](const auto &at) {
+    T ph[NP], lp[NP], cc[NP + 1], rho, hf[NP], gtmp[3];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const T *z = a.pp_out + (size_t)i * a.V;
+      ph[i] = *at.own(z);
+      stencil3m(z, at, ph[i], gtmp, lp[i]);
+    }
+    local_algebra<P, NP>(a, ph, cc, rho, hf);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      T Ci = a.bulk * hf[i];
+#pragma unroll
+      for (int j = 0; j < NP; ++j) Ci -= a.lam[i][j] * lp[j];
+      *at.own(A.C + (size_t)i * a.V) = Ci;
+    }
+  });
+}
+
+template <int P, int NP, bool NU, bool WALL>
+__global__ void __launch_bounds__(NT3, P == LBM_FP64 ? 1 : 2) step3_kernel(const KArgs3<P> A) {
+  typedef typename Prec<P>::T T;
+  const KArgs<P> &a = A.a;
+  for_node3<WALL>(a.nx, a.ny, A.nz, [&](const auto &at) {
+    T ph[NP], gp[NP][3], Cv[NP], cc[NP + 1], rho;
+    T gr[3] = {T(0), T(0), T(0)}, J[3] = {T(0), T(0), T(0)};
+    {
+      T lp[NP], hf[NP];
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        const T *z = a.pp_out + (size_t)i * a.V;
+        ph[i] = *at.own(z);
+        stencil3m(z, at, ph[i], gp[i], lp[i]);
+      }
+      local_algebra<P, NP, !NU>(a, ph, cc, rho, hf);
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        if constexpr (NU) {
+          const T *z = A.C + (size_t)i * a.V;
+          T cg[3], dummy;
+          Cv[i] = *at.own(z);
+          stencil3m(z, at, Cv[i], cg, dummy);
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            J[d] -= a.kmob[i] * cg[d];
+            gr[d] += a.kap[i] * gp[i][d];
+          }
+        } else {
+          T Ci = a.bulk * hf[i];
+#pragma unroll
+          for (int j = 0; j < NP; ++j) Ci -= a.lam[i][j] * lp[j];
+          Cv[i] = Ci;
+        }
+      }
+    }
+    Own3<P, NP> own;
+    load_own3<P, NP>(a, at, own);
+    T F[3], u[3], uu, pr;
+    macros3<P, NP>(a, gp, Cv, rho, gr, own.g, u, F, uu, pr);
+    collide3<P, NP, NU>(a, at, ph, Cv, rho, gr, J, own, u, F, uu, pr, false);
+  });
 }
 
 // Eq. N31 on D3Q15 from three planes (z - 1, z, z + 1) of stride W, pairs of
@@ -656,11 +855,11 @@ __device__ __forceinline__ void stencil3w(const T *pm, const T *p0, const T *pp,
 
 // The step of one node of plane z from the phi window (planes z - 1, z, z + 1
 // with the xy ring, stride SW) and the node's own values (equal densities).
-template <int P, int NP, bool WALL, int SW, int PL>
+template <int P, int NP, int SW, int PL, typename At>
 __device__ __forceinline__ void march3_node(
-    const KArgs<P> &a, int nz, const typename Prec<P>::T (*wm)[PL],
+    const KArgs<P> &a, const At &at, const typename Prec<P>::T (*wm)[PL],
     const typename Prec<P>::T (*w0)[PL], const typename Prec<P>::T (*wp)[PL],
-    int tx, int ty, const Own3<P, NP> &own, size_t q, int gx, int gy, int z) {
+    int tx, int ty, const Own3<P, NP> &own) {
   typedef typename Prec<P>::T T;
   T ph[NP], gp[NP][3], Cv[NP], cc[NP + 1], rho;
   {
@@ -682,84 +881,25 @@ __device__ __forceinline__ void march3_node(
   const T gr[3] = {T(0), T(0), T(0)}, J[3] = {T(0), T(0), T(0)};
   T F[3], u[3], uu, pr;
   macros3<P, NP>(a, gp, Cv, rho, gr, own.g, u, F, uu, pr);
-  collide3<P, NP, false, WALL>(a, nz, ph, Cv, rho, gr, J, own, u, F, uu, pr, q, gx, gy, z);
-}
-
-template <int P, int NP, bool WALL>
-__global__ void __launch_bounds__(MT3, P == LBM_FP64 ? 1 : 2)
-    march3_kernel(const KArgs3<P> A, int zlen) {
-  typedef typename Prec<P>::T T;
-  const KArgs<P> &a = A.a;
-  constexpr int SW = MX3 + 2, SH = MY3 + 2, PL = SW * SH;
-  // the own column's decoded h and g of the plane summed last, then the
-  // window (march3_smem)
-  extern __shared__ __align__(16) unsigned char smem_m3[];
-  T *ocache = (T *)smem_m3;
-  T(*win)[NP][PL] = (T(*)[NP][PL])(smem_m3 + march3_cache_bytes<P, NP>());
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * MX3 + tx;
-  const int nx = a.nx, ny = a.ny, nz = A.nz;
-  const int x0 = blockIdx.x * MX3, y0 = blockIdx.y * MY3;
-  const int zs = blockIdx.z * zlen;
-  const int ze = zs + zlen < nz ? zs + zlen : nz;
-  const int gx = x0 + tx, gy = y0 + ty;
-  const bool col = gx < nx && gy < ny;
-  // window slot of plane z (z >= zs - 1)
-  auto slot = [&](int z) { return (z - zs + 1) % 3; };
-  // phi of plane z on the tile (wrapped where the tile overhangs the grid)
-  // and its xy ring
-  // (the own column's decoded values go to the cache, also on the two
-  // planes outside the slab, where they are not used: a guard there cost
-  // the 16-bit forms 40%)
-  auto plane_phi = [&](int z) {
-    T(*w)[PL] = win[slot(z)];
-    const int zz = wrap(z, nz);
-    {
-      const int cx = wrap(gx, nx), cy = wrap_y<WALL>(gy, ny);
-      const size_t q = ((size_t)zz * ny + cy) * nx + cx;
-      T phv[NP];
-      node_phis3<P, NP, WALL, true>(a, nz, cx, cy, zz, q, phv, ocache + tid, MT3);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) w[i][(ty + 1) * SW + tx + 1] = phv[i];
-    }
-    constexpr int NRING = PL - MT3;
-    static_assert(NRING <= MT3, "one ring position per thread");
-    if (tid < NRING) {
-      int lx, ly;
-      ring_pos_1<MY3>(tid, lx, ly);
-      const int rx = wrap(x0 - 1 + lx, nx), ry = wrap_y<WALL>(y0 - 1 + ly, ny);
-      const size_t q = ((size_t)zz * ny + ry) * nx + rx;
-      T phv[NP];
-      node_phis3<P, NP, WALL>(a, nz, rx, ry, zz, q, phv);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) w[i][ly * SW + lx] = phv[i];
-    }
-  };
-  plane_phi(zs - 1);
-  plane_phi(zs);
-  for (int z = zs; z < ze; ++z) {
-    // this plane's own-node values (decoded when phi of this plane was
-    // summed) first, then phi of the next plane
-    const size_t q = col ? ((size_t)z * ny + gy) * nx + gx : 0;
-    Own3<P, NP> own;
-    load_own3c<P, NP>(a, q, ocache + tid, MT3, own);
-    plane_phi(z + 1);
-    __syncthreads();
-    if (col)
-      march3_node<P, NP, WALL, SW, PL>(a, nz, win[slot(z - 1)], win[slot(z)],
-                                       win[slot(z + 1)], tx, ty, own, q, gx, gy, z);
-    __syncthreads();  // plane z - 1's slot is refilled next
-  }
+  collide3<P, NP, false>(a, at, ph, Cv, rho, gr, J, own, u, F, uu, pr);
 }
 
 // ---------------------------------------------------------------------------
-// The z-marching step with its planes staged by TMA (FP32, N <= 4, nx a
-// multiple of 4): per plane one 4-D box per array, the column with one halo
+// z-marching step kernel (equal densities, FP32, N <= 4, nx a multiple of 4,
+// large grids). A CTA owns a 32 x 8 column of the grid and walks a slab of z
+// planes. phi of plane z + 1 is summed on the column's tile and its xy ring
+// into a rolling window of three planes (z - 1, z, z + 1) in shared memory; the
+// 14 stencil neighbours of a node of plane z then come from the window. The
+// per-node step is the one of tile3_kernel (macros3, collide3). The planes are
+// staged by TMA: per plane one 4-D box per array, the column with one halo
 // row and four halo columns (h^i_k, d^i_0, phi_i(t-1)) or the column alone
 // (g_k, u(t-1)), into two stages; the boxes of plane z + 2 load while plane
 // z + 1's phi is summed and plane z stepped. Ring positions that wrap around
 // the grid (or lie on a wall's ghost row) and columns that overhang it read
-// global memory; everything else comes from the stage, with the same
-// arithmetic as march3_kernel. One CTA of 8 warps per SM.
+// global memory; everything else comes from the stage. One CTA of 8 warps per
+// SM. Stores take their addresses from a plane's uniform offset and a 32-bit
+// offset within it (Off3; index arithmetic was 29% of the instructions): 1386
+// -> 1290 us per step at 256^3, N = 3.
 // ---------------------------------------------------------------------------
 template <int P, int NP> struct March3Stage {
   typedef typename Prec<P>::T T;
@@ -823,6 +963,9 @@ __global__ void __launch_bounds__(MT3, 1)
   const int ze = zs + zlen < nz ? zs + zlen : nz;
   const int gx = x0 + tx, gy = y0 + ty;
   const bool col = gx < nx && gy < ny;
+  const bool at_wall = WALL && (gy == 0 || gy == ny - 1);
+  Off3 oc;
+  oc.set_xy(gx, gy, nx, ny);
   auto slot = [&](int z) { return (z - zs + 1) % 3; };
   // stage and barrier of plane p >= zs; the barrier's k-th completion
   // (parity k & 1) is the k-th plane loaded into that stage
@@ -972,10 +1115,18 @@ __global__ void __launch_bounds__(MT3, 1)
       failed_at = z;
       break;
     }
-    if (col)
-      march3_node<P, NP, WALL, SW, PL>(a, nz, win[slot(z - 1)], win[slot(z)],
-                                       win[slot(z + 1)], tx, ty, own,
-                                       ((size_t)z * ny + gy) * nx + gx, gx, gy, z);
+    if (col) {
+      if (!at_wall) {
+        Off3 o = oc;
+        o.set_z(z, nz, (size_t)nx * ny);
+        march3_node<P, NP, SW, PL>(a, o, win[slot(z - 1)], win[slot(z)], win[slot(z + 1)], tx,
+                                   ty, own);
+      } else {
+        march3_node<P, NP, SW, PL>(
+            a, Nb3<WALL>(gx, gy, z, ((size_t)z * ny + gy) * nx + gx, nx, ny, nz),
+            win[slot(z - 1)], win[slot(z)], win[slot(z + 1)], tx, ty, own);
+      }
+    }
   }
   if (failed_at >= 0 || !ok) {
     // record the timeout and let the loads still in flight land (bounded)
@@ -1095,6 +1246,18 @@ __global__ void init3_pop_kernel(const KArgs3<P> A, const KArgs<LBM_FP64> d,
   }
 }
 
+// Whether the TMA-staged z-marching kernel beats the split step: it reads h
+// once, but needs columns enough to fill the GPU and few idle lanes in them.
+// us per step, march / split, N = 3: 64^3 29.8 / 23.8, 96^3 86.5 / 87.2, 128^3
+// 184 / 199, 160^3 329 / 384, 256^3 1290 / 1538, 40 x 200 x 120 (62% of the
+// columns' lanes) 152 / 114; N = 2: 128^3 133 / 124, 192 x 192 x 200 401 / 424.
+inline bool march3_pays(const Grid &g, int NP) {
+  if (!g.tma3) return false;
+  if (g.march_all) return true;
+  const long long cols = (long long)tiles_x(g.nx) * 32 * ((g.ny + MY3 - 1) / MY3) * MY3;
+  return g.V >= ((size_t)1 << (NP >= 2 ? 20 : 22)) && (long long)g.nx * g.ny * 5 >= cols * 4;
+}
+
 template <int P, int NP, bool NU, bool WALL>
 cudaError_t launch_tile3_t(const Consts &c, const Grid &g, int cur, int mode,
                            const Outputs &o, cudaStream_t s) {
@@ -1102,44 +1265,42 @@ cudaError_t launch_tile3_t(const Consts &c, const Grid &g, int cur, int mode,
   KArgs3<P> A;
   A.a = make_args<P>(c, g, cur, mode, o);
   A.nz = g.nz;
-  if constexpr (!NU) {
-    if (mode == MODE_STEP && g.march3) {
-      // slabs of z planes: enough CTAs to fill the GPU (~1216), at least 8
-      // planes per slab (each slab sums phi on two extra planes)
-      const int txy = tiles_x(g.nx) * ((g.ny + MY3 - 1) / MY3);
-      long long zl = ((long long)g.nz * txy + 1215) / 1216;
-      if (zl < 8) zl = 8;
-      if (zl > g.nz) zl = g.nz;
-      const int zlen = (int)zl;
-      dim3 grid(tiles_x(g.nx), (g.ny + MY3 - 1) / MY3, (g.nz + zlen - 1) / zlen);
-      if constexpr (P == LBM_FP32 && NP <= 3) {
-        if (g.tma3) {
-          typedef March3Stage<P, NP> St;
-          static bool tattr = false;
-          if (!tattr) {
-            cudaError_t e = cudaFuncSetAttribute(march3_tma_kernel<P, NP, WALL>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)St::SMEM);
-            if (e != cudaSuccess) return e;
-            tattr = true;
-          }
-          march3_tma_kernel<P, NP, WALL><<<grid, dim3(MX3, MY3), St::SMEM, s>>>(
-              A, *(const TmaMaps *)&g.tma[cur], zlen);
-          return cudaGetLastError();
+  A.C = (T *)g.scratch;
+  const dim3 tiles(tiles3_x(g.nx), tiles3_y(g.ny), tiles3_z(g.nz)), tblock(BX3, BY3, BZ3);
+  if (mode == MODE_STEP && g.split3) {
+    if constexpr (P == LBM_FP32 && NP <= 3 && !NU) {
+      if (march3_pays(g, NP)) {
+        // slabs of z planes: enough CTAs to fill the GPU (~1216), at least 8
+        // planes per slab (each slab sums phi on two extra planes)
+        const int txy = tiles_x(g.nx) * ((g.ny + MY3 - 1) / MY3);
+        long long zl = ((long long)g.nz * txy + 1215) / 1216;
+        if (zl < 8) zl = 8;
+        if (zl > g.nz) zl = g.nz;
+        const int zlen = (int)zl;
+        dim3 grid(tiles_x(g.nx), (g.ny + MY3 - 1) / MY3, (g.nz + zlen - 1) / zlen);
+        typedef March3Stage<P, NP> St;
+        static bool tattr = false;
+        if (!tattr) {
+          cudaError_t e = cudaFuncSetAttribute(march3_tma_kernel<P, NP, WALL>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)St::SMEM);
+          if (e != cudaSuccess) return e;
+          tattr = true;
         }
+        march3_tma_kernel<P, NP, WALL><<<grid, dim3(MX3, MY3), St::SMEM, s>>>(
+            A, *(const TmaMaps *)&g.tma[cur], zlen);
+        return cudaGetLastError();
       }
-      constexpr size_t msm = march3_smem<P, NP>();
-      static bool mattr = false;
-      if (!mattr) {
-        cudaError_t e = cudaFuncSetAttribute(march3_kernel<P, NP, WALL>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)msm);
-        if (e != cudaSuccess) return e;
-        mattr = true;
-      }
-      march3_kernel<P, NP, WALL><<<grid, dim3(MX3, MY3), msm, s>>>(A, zlen);
-      return cudaGetLastError();
     }
+    phi3_kernel<P, NP, WALL><<<tiles, tblock, 0, s>>>(A);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && NU) {
+      pot3_kernel<P, NP, WALL><<<tiles, tblock, 0, s>>>(A);
+      e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return e;
+    step3_kernel<P, NP, NU, WALL><<<tiles, tblock, 0, s>>>(A);
+    return cudaGetLastError();
   }
   constexpr int RC = NU ? 1 : 0, R = RC + 1;
   constexpr size_t smem = (size_t)NP * ((BX3 + 2 * R) * (BY3 + 2 * R) * (BZ3 + 2 * R) +
@@ -1153,8 +1314,7 @@ cudaError_t launch_tile3_t(const Consts &c, const Grid &g, int cur, int mode,
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  dim3 grid(tiles3_x(g.nx), tiles3_y(g.ny), tiles3_z(g.nz)), block(BX3, BY3, BZ3);
-  tile3_kernel<P, NP, NU, WALL><<<grid, block, smem, s>>>(A);
+  tile3_kernel<P, NP, NU, WALL><<<tiles, tblock, smem, s>>>(A);
   return cudaGetLastError();
 }
 

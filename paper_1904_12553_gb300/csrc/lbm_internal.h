@@ -75,8 +75,10 @@ struct Grid {
   int grad_scheme;  // 0: central (Eq. N31a), 1: mixed (Eq. N40)
   bool use_tma;     // pipelined kernel usable for this grid
   bool step64;      // D2Q9 step by the FP64 kernels (lbm_step64.cuh)
-  bool march3;      // D3Q15 step by the z-marching kernel
-  bool tma3;        // ... with its planes staged by TMA (tma[] holds 4-D maps)
+  bool split3;      // D3Q15 step by the split or z-marching kernels
+  bool march3;      // ... with equal densities
+  bool tma3;        // ... FP32 z-marching kernel prepared (tma[] holds 4-D maps)
+  bool march_all;   // ... and taken at every size (LBM_NPHASE_KERNEL=march)
   TmaMaps tma[2];   // its descriptors, input buffer 0 or 1
 };
 
