@@ -284,15 +284,16 @@ int64_t lbm_nphase_steps_taken(const lbm_nphase_t *h);
 
 /* Which kernels lbm_nphase_step has for this handle: 1 the TMA-pipelined
  * D2Q9 kernel (FP32 and 16-bit forms, equal pure-phase densities, nx a
- * multiple of 8), 2 the D3Q15 step split into a phi and a step kernel (equal
+ * multiple of 8; FP32 grids of up to 608 tiles of 32 x 8 nodes run the
+ * generic tile kernel, which is faster there), 2 the D3Q15 step split into a phi and a step kernel (equal
  * densities, every storage form), 3 the same and the z-marching D3Q15 kernel
  * with TMA-staged planes for large boxes (FP32, equal densities, N <= 4, nx a
  * multiple of 4), 0 the others (D2Q9: FP64 kernels or the generic tile
  * kernel; D3Q15, unequal densities: split into phi, C_i and step kernels).
  * Setting the environment variable LBM_NPHASE_KERNEL before
  * lbm_nphase_create to "generic" selects the generic tile kernels everywhere,
- * to "march" the z-marching kernel at every size of case 3. All compute the
- * same step. */
+ * to "pipelined" the TMA kernels at every size of cases 1 and 3. All compute
+ * the same step. */
 int lbm_nphase_uses_pipelined_kernel(const lbm_nphase_t *h);
 
 /* Self-test of the timeout path (not part of the paper). Launches, on the

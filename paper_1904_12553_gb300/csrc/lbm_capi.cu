@@ -508,7 +508,7 @@ lbm_status lbm_nphase_create(const lbm_nphase_params *p, void *ws,
              (size_t)p->nx * p->ny * sT < ((size_t)1 << 32);
   g.march3 = g.split3 && !h->nonunif;
   const char *kv = getenv("LBM_NPHASE_KERNEL");
-  g.march_all = kv && strcmp(kv, "march") == 0;
+  g.tma_all = kv && strcmp(kv, "pipelined") == 0;
   g.tma3 = g.march3 && h->prec == LBM_FP32 &&
            lbm::encode_tma3_f32(k, g, tensor_map_encoder());
   if (tma_allowed() && !h->nonunif && p->grad_scheme == 0 && p->lattice == 0) {

@@ -1253,7 +1253,7 @@ __global__ void init3_pop_kernel(const KArgs3<P> A, const KArgs<LBM_FP64> d,
 // columns' lanes) 152 / 114; N = 2: 128^3 133 / 124, 192 x 192 x 200 401 / 424.
 inline bool march3_pays(const Grid &g, int NP) {
   if (!g.tma3) return false;
-  if (g.march_all) return true;
+  if (g.tma_all) return true;
   const long long cols = (long long)tiles_x(g.nx) * 32 * ((g.ny + MY3 - 1) / MY3) * MY3;
   return g.V >= ((size_t)1 << (NP >= 2 ? 20 : 22)) && (long long)g.nx * g.ny * 5 >= cols * 4;
 }

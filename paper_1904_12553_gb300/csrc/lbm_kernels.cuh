@@ -767,8 +767,24 @@ __device__ __forceinline__ void phi_global(const KArgs<P> &a, int sx, int sy,
 // time step; MODE_MOMENTS: write the macroscopic fields; MODE_DIAG: per-CTA
 // partial sums of the diagnostics).
 // ---------------------------------------------------------------------------
+// Resident CTAs the FP32 kernel is compiled for, and whether a node's NS
+// populations and u(t-1) are loaded before the halo ring (one memory latency
+// instead of two: what counts on a grid of one wave of tiles) where registers
+// are left for them. us per step in 2 / 3 / 4 CTAs (e: loaded early): N = 3,
+// 256^2 4.49e / 4.50e / 4.69e (4.87 before); N = 5, 256^2 6.23e / 7.05e /
+// 13.4e (6.43 before), 512^2 23.2e / 24.1e; N = 4, 1501 x 997 116e / 105.7e,
+// 105.9 / 101 (104 before); N = 3 unequal densities, 1024^2 74e / 65e, 60.5 /
+// 56.9 (62.4 before), 400 x 200 8.2e / 7.0e, 6.9 / 7.1 (7.1 before); Eq. N40,
+// N = 4, 512^2 18.3e / 17.1e, 17.3 / 18.0 (17.2 before).
+template <int P, int NP, bool NU, bool G40> struct TileMin {
+  static constexpr bool F32 = P == LBM_FP32;
+  static constexpr bool EARLY = F32 && !NU && (NP == 2 || NP == 4);
+  static constexpr int CTAS = !F32 ? 0 : (NP == 4 ? 2 : (!G40 && (NU || NP != 2) ? 4 : 3));
+};
+
 template <int P, int NP, bool NU, bool WALL, bool G40>
-__global__ void __launch_bounds__(NT) tile_kernel(const KArgs<P> a) {
+__global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel(const KArgs<P> a) {
+  constexpr bool EARLY = TileMin<P, NP, NU, G40>::EARLY;
   typedef typename Prec<P>::T T;
   constexpr int RG = G40 ? 2 : 1;          // reach of a gradient stencil
   constexpr int RC = NU ? RG : 0;          // C ring radius (for grad C)
@@ -801,6 +817,21 @@ __global__ void __launch_bounds__(NT) tile_kernel(const KArgs<P> a) {
           node_phi<P>(hreg[i][0], &hreg[i][1], pp, perr[i], a.sh_ld);
     }
   }
+  const size_t q = (size_t)(active ? gy : 0) * nx + (active ? gx : 0);
+  T g[9], up[2];
+  auto load_rest = [&] {  // the node's NS populations and u(t-1)
+    if (active) {
+      load_g_node<P, WALL>(a, gx, gy, q, g);
+    } else {
+#pragma unroll
+      for (int k = 1; k < 9; ++k) g[k] = T(0);
+    }
+    if (EARLY) {
+      up[0] = ldg(a.u_in + q);
+      up[1] = ldg(a.u_in + V + q);
+    }
+  };
+  if (EARLY) load_rest();
   // 2. Halo ring.
   constexpr int NRING = SW * SH - BX * BY;
   for (int r = tid; r < NRING; r += NT) {
@@ -848,14 +879,7 @@ __global__ void __launch_bounds__(NT) tile_kernel(const KArgs<P> a) {
   }
 
   // 4. Own node: stencils, C_i, forces, u, p.
-  const size_t q = (size_t)(active ? gy : 0) * nx + (active ? gx : 0);
-  T g[9];
-  if (active) {
-    load_g_node<P, WALL>(a, gx, gy, q, g);
-  } else {
-#pragma unroll
-    for (int k = 1; k < 9; ++k) g[k] = T(0);
-  }
+  if (!EARLY) load_rest();
   NodeMac<P, NP> m;
   node_macros<P, NP, NU, SW, CW, G40>(a, &sphi[0][0], SH * SW, &sC[0][0],
                                       CH * CW, ty + R, tx + R, ty + RC,
@@ -905,8 +929,11 @@ __global__ void __launch_bounds__(NT) tile_kernel(const KArgs<P> a) {
   T pp[NP];
 #pragma unroll
   for (int i = 0; i < NP; ++i) pp[i] = ldg(a.pp_in + (size_t)i * V + q);
-  collide_stream<P, NP, NU, WALL>(a, m, hreg, perr, g, pp, a.u_in[q],
-                                  a.u_in[V + q], gx, gy);
+  if (!EARLY) {
+    up[0] = a.u_in[q];
+    up[1] = a.u_in[V + q];
+  }
+  collide_stream<P, NP, NU, WALL>(a, m, hreg, perr, g, pp, up[0], up[1], gx, gy);
 }
 
 // ---------------------------------------------------------------------------
@@ -1635,6 +1662,17 @@ namespace lbm {
 // ---------------------------------------------------------------------------
 // Host-side launchers for one precision.
 // ---------------------------------------------------------------------------
+// FP32 grids of up to four waves of tiles on 152 SMs take the generic kernel:
+// its CTAs start their loads at once and overlap on an SM, where the pipelined
+// kernel's single CTA fetches its tensor maps and fills its stages first. us
+// per step, pipelined / generic: N = 3, 64^2 4.04 / 3.35, 256^2 5.29 / 4.45,
+// 384^2 (576 tiles) 7.88 / 7.65; N = 5, 256^2 8.40 / 6.23, 384^2 13.1 / 11.0,
+// 512^2 (1024 tiles) 20.8 / 23.2. The 16-bit forms' decode makes the generic
+// kernel slower at every size (BF16 N = 3, 128^2 4.9 / 6.6).
+template <int P> inline bool pipelined_pays(const Grid &g) {
+  return P != LBM_FP32 || g.tma_all || (long long)tiles_x(g.nx) * tiles_y(g.ny) > 4 * 152;
+}
+
 template <int P, int NP, bool NU, bool WALL>
 cudaError_t launch_tile_t(const Consts &c, const Grid &g, int cur, int mode,
                           const Outputs &o, cudaStream_t s) {
@@ -1642,7 +1680,7 @@ cudaError_t launch_tile_t(const Consts &c, const Grid &g, int cur, int mode,
     if (mode == MODE_STEP && g.step64) return launch_step64<NP, NU, WALL>(c, g, cur, s);
   const KArgs<P> a = make_args<P>(c, g, cur, mode, o);
   if constexpr (P != LBM_FP64 && !NU) {
-    if (mode == MODE_STEP && g.use_tma && g.grad_scheme == 0) {
+    if (mode == MODE_STEP && g.use_tma && g.grad_scheme == 0 && pipelined_pays<P>(g)) {
       typedef TmaStage<P, NP> St;
       constexpr int TBY = TmaGeom<P>::TBY;
       const bool whole = g.nx % BX == 0 && g.ny % TBY == 0 && g.nx > BX && g.ny > TBY;

@@ -43,7 +43,7 @@ def test_unequal_densities_match_generic(N, prec, shape, wall):
 
 def march(w, steps):
     from paper_1904_12553_gb300 import Solver
-    os.environ["LBM_NPHASE_KERNEL"] = "march"
+    os.environ["LBM_NPHASE_KERNEL"] = "pipelined"
     try:
         s = Solver(w.params)
     finally:
