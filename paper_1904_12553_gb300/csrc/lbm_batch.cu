@@ -43,7 +43,7 @@ __device__ __forceinline__ void tile_step_body(const KArgs<P> &a, int x0, int y0
   T hreg[NP][9], perr[NP];
   {
     const int sx = wrap(gx, nx), sy = wrap_y<WALL>(gy, ny);
-    const size_t q = (size_t)sy * nx + sx;
+    const size_t q = (size_t)sy * a.px + sx;
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
       hreg[i][0] = ldg(a.h0_in + (size_t)i * V + q);
@@ -63,7 +63,7 @@ __device__ __forceinline__ void tile_step_body(const KArgs<P> &a, int x0, int y0
   }
   __syncthreads();
   if (active) {
-    const size_t q = (size_t)gy * nx + gx;
+    const size_t q = (size_t)gy * a.px + gx;
     T g[9], pp[NP];
 #pragma unroll
     for (int k = 1; k < 9; ++k) g[k] = load_gm<P>(a, k, q);
@@ -247,6 +247,46 @@ __device__ __forceinline__ void batch_tma_phi(const KArgs<LBM_FP32> &a,
   const T *spp = (const T *)(st + St::HM + St::H0);
   const Sm *sgm = (const Sm *)(st + St::HM + St::H0 + St::PP);
   const int gx = x0 + tx, gy = y0 + ty;
+  // phi at tile position (lx, ly), at most one beyond the grid
+  auto edge_phi = [&](int lx, int ly) {
+    const int rx = x0 - 1 + lx;
+    // a wall's ghost row is the adjacent row of the box
+    const int ry = WALL ? wrap_y<WALL>(y0 - 1 + ly, ny) : y0 - 1 + ly, by = ry - y0 + 1;
+    const bool inx = rx >= 0 && rx < nx, iny = ry >= 0 && ry < ny;
+    // phi of one position from staged populations: hmb, h0b, ppb are the
+    // moving, rest and phi(t-1) planes with plane strides pm, pr; om, orr
+    // the position's offset in them
+    auto staged_phi = [&](const Sm *hmb, const T *h0b, const T *ppb, int pm, int pr,
+                          int om, int orr) {
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        T mov[8], e;
+#pragma unroll
+        for (int k = 1; k < 9; ++k) mov[k - 1] = to_T(hmb[(i * 8 + k - 1) * pm + om]);
+        sphi[i * PL + ly * SW + lx] =
+            node_phi<LBM_FP32>(h0b[i * pr + orr], mov, ppb[i * pr + orr], e, a.sh_ld);
+      }
+    };
+    const unsigned char *w = st + St::BASE;
+    if (inx && iny) {
+      staged_phi(shm, sh0, spp, BG::HB * BG::WM, BG::HB * BG::WR,
+                 by * BG::WM + lx - 1 + BG::HXM, by * BG::WR + lx - 1 + BG::HXR);
+    } else if (iny && ((rx < 0 && wx == 1) || (rx >= nx && wx == 2))) {
+      // the staged wrapped column
+      const int c = rx < 0 ? BG::HXR - 1 : 0;
+      staged_phi((const Sm *)w, (const T *)(w + St::XHM), (const T *)(w + St::XHM + St::XH0),
+                 BG::HB * BG::HXM, BG::HB * BG::HXR, by * BG::HXM + c, by * BG::HXR + c);
+    } else if (inx && ((ry < 0 && wy == 1) || (ry >= ny && wy == 2))) {
+      // the staged wrapped row
+      w += St::XHM + St::XH0 + St::XPP;
+      staged_phi((const Sm *)w, (const T *)(w + St::YHM), (const T *)(w + St::YHM + St::YH0),
+                 BG::WM, BG::WR, lx - 1 + BG::HXM, lx - 1 + BG::HXR);
+    } else {
+      // corners, grids one tile wide or high
+      phi_global<LBM_FP32, NP, WALL>(a, wrap(rx, nx), wrap_y<WALL>(ry, ny), sphi, PL,
+                               ly * SW + lx);
+    }
+  };
   if (gx < nx && gy < ny) {
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
@@ -264,9 +304,9 @@ __device__ __forceinline__ void batch_tma_phi(const KArgs<LBM_FP32> &a,
     const T *sup = (const T *)(st + St::HM + St::H0 + St::PP + St::GM);
     r.up[0] = sup[ty * BX + tx];
     r.up[1] = sup[(TBY + ty) * BX + tx];
-  } else {
-    phi_global<LBM_FP32, NP, WALL>(a, wrap(gx, nx), wrap_y<WALL>(gy, ny), sphi, PL,
-                             (ty + 1) * SW + tx + 1);
+  } else if (gx <= nx && gy <= ny) {
+    // the position one beyond the grid in a tile that overhangs it
+    edge_phi(tx + 1, ty + 1);
   }
   // The ring's positions go to warps 1..3 (threads 32 .. 32 + NRING - 1):
   // warp 0 holds the thread that fetches the next item and issues its
@@ -276,43 +316,7 @@ __device__ __forceinline__ void batch_tma_phi(const KArgs<LBM_FP32> &a,
   if (tid >= 32 && tid < 32 + NRING) {
     int lx, ly;
     ring_pos_1<TBY>(tid - 32, lx, ly);
-    const int rx = x0 - 1 + lx, ry = y0 - 1 + ly;
-    const bool inx = rx >= 0 && rx < nx, iny = ry >= 0 && ry < ny;
-    // phi of one ring position from staged populations: hmb, h0b, ppb are
-    // the moving, rest and phi(t-1) planes with plane strides pm, pr; om,
-    // orr the position's offset in them
-    auto staged_phi = [&](const Sm *hmb, const T *h0b, const T *ppb, int pm, int pr,
-                          int om, int orr) {
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        T mov[8], e;
-#pragma unroll
-        for (int k = 1; k < 9; ++k) mov[k - 1] = to_T(hmb[(i * 8 + k - 1) * pm + om]);
-        sphi[i * PL + ly * SW + lx] =
-            node_phi<LBM_FP32>(h0b[i * pr + orr], mov, ppb[i * pr + orr], e, a.sh_ld);
-      }
-    };
-    const unsigned char *w = st + St::BASE;
-    if (inx && (iny || WALL)) {
-      // in the box; a wall's ghost row is the adjacent row of the box
-      const int by = WALL ? wrap_y<WALL>(ry, ny) - y0 + 1 : ly;
-      staged_phi(shm, sh0, spp, BG::HB * BG::WM, BG::HB * BG::WR,
-                 by * BG::WM + lx - 1 + BG::HXM, by * BG::WR + lx - 1 + BG::HXR);
-    } else if (iny && ((rx < 0 && wx == 1) || (rx >= nx && wx == 2))) {
-      // the staged wrapped column
-      const int c = rx < 0 ? BG::HXR - 1 : 0;
-      staged_phi((const Sm *)w, (const T *)(w + St::XHM), (const T *)(w + St::XHM + St::XH0),
-                 BG::HB * BG::HXM, BG::HB * BG::HXR, ly * BG::HXM + c, ly * BG::HXR + c);
-    } else if (inx && ((ry < 0 && wy == 1) || (ry >= ny && wy == 2))) {
-      // the staged wrapped row
-      w += St::XHM + St::XH0 + St::XPP;
-      staged_phi((const Sm *)w, (const T *)(w + St::YHM), (const T *)(w + St::YHM + St::YH0),
-                 BG::WM, BG::WR, lx - 1 + BG::HXM, lx - 1 + BG::HXR);
-    } else {
-      // corners and ragged tails
-      phi_global<LBM_FP32, NP, WALL>(a, wrap(rx, nx), wrap_y<WALL>(ry, ny), sphi, PL,
-                               ly * SW + lx);
-    }
+    if (x0 - 1 + lx <= nx && y0 - 1 + ly <= ny) edge_phi(lx, ly);
   }
 }
 
@@ -527,7 +531,7 @@ lbm_status bfail(lbm_nphase_batch_t *b, cudaError_t e) {
 }
 
 size_t case_bytes(const lbm_nphase_params &p) {
-  return align256b(lbm_nphase_workspace_bytes(&p));
+  return align256b(lbm::workspace_bytes(&p, false));
 }
 
 size_t tiles_for(const lbm_nphase_params &p, int tby) {
@@ -636,8 +640,8 @@ lbm_status build_schedule(lbm_nphase_batch_t *b, lbm_nphase_batch_schedule s) {
       const int x0 = (t % ntx) * lbm::BX, y0 = (t / ntx) * tby;
       const int nx = h->prm.nx, ny = h->prm.ny;
       // wrapped halo column / row staged with an edge tile (periodic axes)
-      const int wx = x0 == 0 ? 1 : (x0 + lbm::BX == nx ? 2 : 0);
-      const int wy = h->wall ? 0 : (y0 == 0 ? 1 : (y0 + tby == ny ? 2 : 0));
+      const int wx = x0 == 0 ? 1 : (x0 + lbm::BX >= nx ? 2 : 0);
+      const int wy = h->wall ? 0 : (y0 == 0 ? 1 : (y0 + tby >= ny ? 2 : 0));
       titems[i] = {items[i].x, x0, y0, h->k.NP * 2 + (h->wall ? 1 : 0), wx, wy,
                    wx == 1 ? nx - lbm::TmaGeom<LBM_FP32>::HXR : 0, wy == 1 ? ny - 1 : 0};
     }
@@ -736,7 +740,7 @@ lbm_status lbm_nphase_batch_create(const lbm_nphase_params *params, int ncases,
   for (int c = 0; c < ncases && st == LBM_OK; ++c) {
     lbm_nphase_t *h = nullptr;
     const size_t cb = case_bytes(params[c]);
-    st = lbm_nphase_create(&params[c], base + off, cb, stream, &h);
+    st = lbm::create(&params[c], base + off, cb, stream, false, &h);
     if (st == LBM_OK) b->cases.push_back(h);
     off += cb;
     items += tiles_for(params[c], 4);

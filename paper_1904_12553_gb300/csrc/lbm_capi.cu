@@ -182,8 +182,21 @@ int uplanes(const lbm_nphase_params *p) {
   return dims(p) + (p->precision == LBM_MIX_BF16 || p->precision == LBM_MIX_FP16 ? 1 : 0);
 }
 
-Layout layout(const lbm_nphase_params *p) {
-  const size_t V = (size_t)p->nx * p->ny * depth(p);
+// Row pitch of the state's planes. The pipelined D2Q9 kernels need rows of
+// whole 16 bytes: grids they can serve (FP32 and 16-bit forms, equal
+// densities, central scheme) are padded to a multiple of 8 nodes, at most 7
+// nodes per row. FP32, us per step on the generic kernel, dense -> padded:
+// see pipelined_pays.
+int pitch(const lbm_nphase_params *p, bool pad) {
+  if (!pad || p->lattice != 0 || p->precision != LBM_FP32 || p->grad_scheme != 0) return p->nx;
+  for (int k = 1; k < p->N; ++k)
+    if (p->rho[k] != p->rho[0]) return p->nx;
+  return (p->nx + 7) / 8 * 8;
+}
+
+Layout layout(const lbm_nphase_params *p, bool pad) {
+  const size_t Vd = (size_t)p->nx * p->ny * depth(p);
+  const size_t V = (size_t)pitch(p, pad) * p->ny * depth(p);
   const int NP = p->N - 1, QM = moving_dirs(p), D = dims(p), UP = uplanes(p);
   const size_t sT = p->precision == LBM_FP64 ? 8 : 4;
   const size_t sS = p->precision == LBM_FP64 ? 8 : (p->precision == LBM_FP32 ? 4 : 2);
@@ -195,7 +208,7 @@ Layout layout(const lbm_nphase_params *p) {
   L.gm = off;       off += 2 * align256(QM * V * sS);
   L.phi_prev = off; off += 2 * align256(NP * V * sT);
   L.u_prev = off;   off += 2 * align256(UP * V * sT);
-  L.stage = off;    off += align256((p->N + D) * V * 8);
+  L.stage = off;    off += align256((p->N + D) * Vd * 8);
   L.red = off;      off += align256(tiles * (p->N + 2) * 8);
   L.red_out = off;  off += align256(8 * 8);
   L.err = off;      off += align256(sizeof(int));
@@ -408,19 +421,29 @@ lbm_status lbm_nphase_derive(const lbm_nphase_params *p, lbm_nphase_model *out) 
 }
 
 size_t lbm_nphase_workspace_bytes(const lbm_nphase_params *p) {
-  if (validate(p) != LBM_OK) return 0;
-  return layout(p).total;
+  return lbm::workspace_bytes(p, true);
 }
 
 lbm_status lbm_nphase_create(const lbm_nphase_params *p, void *ws,
                              size_t bytes, void *stream, lbm_nphase_t **out) {
+  return lbm::create(p, ws, bytes, stream, true, out);
+}
+
+}  // extern "C"
+
+size_t lbm::workspace_bytes(const lbm_nphase_params *p, bool pad) {
+  return validate(p) == LBM_OK ? layout(p, pad).total : 0;
+}
+
+lbm_status lbm::create(const lbm_nphase_params *p, void *ws, size_t bytes, void *stream, bool pad,
+                       lbm_nphase_t **out) {
   if (!out) return LBM_EINVAL;
   *out = nullptr;
   lbm_nphase_model m;
   lbm_status st = lbm_nphase_derive(p, &m);
   if (st != LBM_OK) return st;
   if (!ws || ((uintptr_t)ws & 255u)) return LBM_EINVAL;
-  const Layout L = layout(p);
+  const Layout L = layout(p, pad);
   if (bytes < L.total) return LBM_ENOMEM;
   lbm_nphase_t *h = new (std::nothrow) lbm_nphase_t;
   if (!h) return LBM_ENOMEM;
@@ -477,7 +500,8 @@ lbm_status lbm_nphase_create(const lbm_nphase_params *p, void *ws,
   g.ny = p->ny;
   g.nz = depth(p);
   g.lattice = p->lattice;
-  g.V = (size_t)p->nx * p->ny * g.nz;
+  g.px = pitch(p, pad);
+  g.V = (size_t)g.px * p->ny * g.nz;
   char *base = (char *)ws;
   const size_t sT = h->prec == LBM_FP64 ? 8 : 4;
   const size_t sS = h->prec == LBM_FP64 ? 8 : (h->prec == LBM_FP32 ? 4 : 2);
@@ -524,6 +548,8 @@ lbm_status lbm_nphase_create(const lbm_nphase_params *p, void *ws,
   return LBM_OK;
 }
 
+extern "C" {
+
 lbm_status lbm_nphase_init(lbm_nphase_t *h, const double *c, const double *u,
                            double p0) {
   return lbm::init_at(h, c, u, p0, 0);
@@ -534,7 +560,7 @@ lbm_status lbm_nphase_init(lbm_nphase_t *h, const double *c, const double *u,
 lbm_status lbm::init_at(lbm_nphase_t *h, const double *c, const double *u,
                         double p0, int cur) {
   if (!h || !c || !isfinite(p0) || (cur != 0 && cur != 1)) return LBM_EINVAL;
-  const size_t V = h->g.V;
+  const size_t V = (size_t)h->g.nx * h->g.ny * h->g.nz;
   const int N = h->prm.N;
   const double *dc = c, *du = u;
   cudaError_t e;
@@ -658,22 +684,37 @@ static_assert(sizeof(StateHeader) == 64, "state header");
 
 struct Part {
   void *dev;
-  size_t bytes;
+  size_t planes, es;  // planes of ny nz rows of nx values of es bytes
 };
 
 int state_parts(const lbm_nphase_t *h, Part out[5]) {
-  const size_t V = h->g.V;
-  const int n = h->prm.N - 1;
+  const size_t n = h->prm.N - 1;
   const size_t sT = h->prec == LBM_FP64 ? 8 : 4;
   const size_t sS = h->prec == LBM_FP64 ? 8 : (h->prec == LBM_FP32 ? 4 : 2);
   const int c = h->cur;
-  const int QM = moving_dirs(&h->prm), UP = uplanes(&h->prm);
-  out[0] = {h->g.h0[c], n * V * sT};
-  out[1] = {h->g.hm[c], n * QM * V * sS};
-  out[2] = {h->g.gm[c], QM * V * sS};
-  out[3] = {h->g.phi_prev[c], n * V * sT};
-  out[4] = {h->g.u_prev[c], UP * V * sT};
+  const size_t QM = moving_dirs(&h->prm), UP = uplanes(&h->prm);
+  out[0] = {h->g.h0[c], n, sT};
+  out[1] = {h->g.hm[c], n * QM, sS};
+  out[2] = {h->g.gm[c], QM, sS};
+  out[3] = {h->g.phi_prev[c], n, sT};
+  out[4] = {h->g.u_prev[c], UP, sT};
   return 5;
+}
+
+size_t part_bytes(const lbm_nphase_t *h, const Part &p) {
+  return p.planes * h->g.nx * h->g.ny * h->g.nz * p.es;
+}
+
+// Copies a part to or from the blob's dense rows.
+cudaError_t copy_part(const lbm_nphase_t *h, const Part &p, void *blob, bool to_blob,
+                      cudaMemcpyKind kind) {
+  const size_t row = (size_t)h->g.nx * p.es, pitch = (size_t)h->g.px * p.es;
+  if (row == pitch)
+    return to_blob ? cudaMemcpyAsync(blob, p.dev, part_bytes(h, p), kind, h->stream)
+                   : cudaMemcpyAsync(p.dev, blob, part_bytes(h, p), kind, h->stream);
+  const size_t rows = p.planes * h->g.ny * h->g.nz;
+  return to_blob ? cudaMemcpy2DAsync(blob, row, p.dev, pitch, row, rows, kind, h->stream)
+                 : cudaMemcpy2DAsync(p.dev, pitch, blob, row, row, rows, kind, h->stream);
 }
 }  // namespace
 
@@ -681,7 +722,8 @@ size_t lbm_nphase_state_bytes(const lbm_nphase_t *h) {
   if (!h) return 0;
   Part parts[5];
   size_t b = sizeof(StateHeader);
-  for (int i = 0; i < state_parts(h, parts); ++i) b += parts[i].bytes;
+  const int np = state_parts(h, parts);
+  for (int i = 0; i < np; ++i) b += part_bytes(h, parts[i]);
   return b;
 }
 
@@ -708,11 +750,10 @@ lbm_status lbm_nphase_get_state(lbm_nphase_t *h, void *dst, size_t bytes) {
                                   h->stream);
   Part parts[5];
   char *p = (char *)dst + sizeof(hd);
-  for (int i = 0; i < state_parts(h, parts) && e == cudaSuccess; ++i) {
-    e = cudaMemcpyAsync(p, parts[i].dev, parts[i].bytes,
-                        dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                        h->stream);
-    p += parts[i].bytes;
+  const int np = state_parts(h, parts);
+  for (int i = 0; i < np && e == cudaSuccess; ++i) {
+    e = copy_part(h, parts[i], p, true, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost);
+    p += part_bytes(h, parts[i]);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e);
@@ -736,12 +777,11 @@ lbm_status lbm_nphase_set_state(lbm_nphase_t *h, const void *src, size_t bytes) 
     return LBM_EINVAL;
   h->cur = 0;
   Part parts[5];
-  const char *p = (const char *)src + sizeof(hd);
-  for (int i = 0; i < state_parts(h, parts) && e == cudaSuccess; ++i) {
-    e = cudaMemcpyAsync(parts[i].dev, p, parts[i].bytes,
-                        dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                        h->stream);
-    p += parts[i].bytes;
+  char *p = (char *)src + sizeof(hd);
+  const int np = state_parts(h, parts);
+  for (int i = 0; i < np && e == cudaSuccess; ++i) {
+    e = copy_part(h, parts[i], p, false, dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice);
+    p += part_bytes(h, parts[i]);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(h->g.err, 0, sizeof(int), h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -756,7 +796,7 @@ lbm_status lbm_nphase_moments(lbm_nphase_t *h, double *phi, double *c,
                               double *u, double *p, double *rho) {
   if (!h) return LBM_EINVAL;
   if (!h->initialized) return LBM_ESTATE;
-  const size_t V = h->g.V;
+  const size_t V = (size_t)h->g.nx * h->g.ny * h->g.nz;
   const int N = h->prm.N;
   double *ptr[5] = {phi, c, u, p, rho};
   const int nf[5] = {N - 1, N, dims(&h->prm), 1, 1};
@@ -834,7 +874,7 @@ lbm_status lbm_nphase_diagnostics(lbm_nphase_t *h, double *mass, double *ke,
 
 int lbm_nphase_uses_pipelined_kernel(const lbm_nphase_t *h) {
   if (!h) return 0;
-  return h->g.use_tma ? 1 : (h->g.tma3 ? 3 : (h->g.march3 ? 2 : 0));
+  return h->g.use_tma && h->g.nx % 8 == 0 ? 1 : (h->g.tma3 ? 3 : (h->g.march3 ? 2 : 0));
 }
 
 int64_t lbm_nphase_steps_taken(const lbm_nphase_t *h) { return h ? h->steps : 0; }

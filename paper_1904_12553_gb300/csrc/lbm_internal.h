@@ -60,7 +60,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType,
 struct Grid {
   int nx, ny, nz;   // nz = 1 for D2Q9
   int lattice;      // 0 D2Q9, 1 D3Q15
-  size_t V;
+  int px;           // row pitch in nodes (nx, or nx rounded up to 8)
+  size_t V;         // plane stride px * ny * nz
   void *h0[2];      // rest slots: h^i_0 (FP64) or h^i_0 - phi_i(t-1): [N-1][V]
   void *hm[2];      // moving populations h^i_k, k = 1..8: [N-1][8][V]
   void *gm[2];      // NS populations g_k, k = 1..8: [8][V]
@@ -154,4 +155,9 @@ namespace lbm {
 // so that grids stepped together keep the same buffer parity.
 lbm_status init_at(lbm_nphase_t *h, const double *c, const double *u,
                    double p0, int cur);
+// lbm_nphase_create, with rows padded to a multiple of 8 nodes where the
+// pipelined kernels use that (single grids), or dense (the cases of a batch).
+lbm_status create(const lbm_nphase_params *p, void *ws, size_t bytes, void *stream, bool pad,
+                  lbm_nphase_t **out);
+size_t workspace_bytes(const lbm_nphase_params *p, bool pad);
 }  // namespace lbm

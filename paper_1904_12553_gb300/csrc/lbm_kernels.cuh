@@ -119,8 +119,8 @@ template <typename S> __device__ __forceinline__ S to_S(double v) { return v; }
 template <int P> struct alignas(16) KArgs {  // 16: bulk-copy granule
   typedef typename Prec<P>::T T;
   typedef typename Prec<P>::Sm Sm;
-  int nx, ny;
-  size_t V;
+  int nx, ny, px;  // px: row pitch of the state's planes (nodes)
+  size_t V;        // plane stride, px ny
   const T *h0_in;
   const Sm *hm_in, *gm_in;
   T *h0_out;
@@ -145,6 +145,7 @@ KArgs<P> make_args(const Consts &c, const Grid &g, int cur, int mode,
   KArgs<P> a;
   a.nx = g.nx;
   a.ny = g.ny;
+  a.px = g.px;
   a.V = g.V;
   a.h0_in = (const T *)g.h0[cur];
   a.hm_in = (const Sm *)g.hm[cur];
@@ -264,7 +265,7 @@ __device__ __forceinline__ double g_refp(double cu, double ux, double uy,
 // (and in y without walls); behind a wall, (x, y) itself.
 template <bool WALL>
 __device__ __forceinline__ size_t source_node(int x, int y, int k, int nx,
-                                              int ny) {
+                                              int ny, int px) {
   int sx = x - cx_of(k), sy = y - cy_of(k);
   if (WALL && (sy < 0 || sy >= ny)) {
     sx = x;
@@ -272,7 +273,7 @@ __device__ __forceinline__ size_t source_node(int x, int y, int k, int nx,
   }
   sx = sx < 0 ? sx + nx : (sx >= nx ? sx - nx : sx);
   sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
-  return (size_t)sy * nx + sx;
+  return (size_t)sy * px + sx;
 }
 
 // Moving populations of phase i (mov[0..7] = h_1..8) and the NS populations
@@ -286,7 +287,7 @@ __device__ __forceinline__ void load_h_node(const KArgs<P> &a, int i, int x,
   for (int k = 1; k < 9; ++k) {
     T v = load_hm<P>(a, i, k, q);
     if constexpr (Prec<P>::REF) {
-      const size_t qs = source_node<WALL>(x, y, k, a.nx, a.ny);
+      const size_t qs = source_node<WALL>(x, y, k, a.nx, a.ny, a.px);
       const T cu = cdotu(k, ldg(a.u_in + qs), ldg(a.u_in + a.V + qs));
       v = __fadd_rn(v, adv_units(cu, ldg(a.pp_in + (size_t)i * a.V + qs),
                                  T(3) * a.sh_st));
@@ -302,7 +303,7 @@ __device__ __forceinline__ void load_g_node(const KArgs<P> &a, int x, int y,
   for (int k = 1; k < 9; ++k) {
     T v = load_gm<P>(a, k, q);
     if constexpr (Prec<P>::REF) {
-      const size_t qs = source_node<WALL>(x, y, k, a.nx, a.ny);
+      const size_t qs = source_node<WALL>(x, y, k, a.nx, a.ny, a.px);
       const T sux = ldg(a.u_in + qs), suy = ldg(a.u_in + a.V + qs),
               spr = ldg(a.u_in + 2 * a.V + qs);
       v = __fadd_rn(v, g_refp(cdotu(k, sux, suy), sux, suy, spr, a.rho_base * a.sg_st,
@@ -573,7 +574,7 @@ __device__ __forceinline__ void collide_stream(
   typedef typename Prec<P>::T T;
   const int nx = a.nx, ny = a.ny;
   const size_t V = a.V;
-  const size_t q = (size_t)gy * nx + gx;
+  const size_t q = (size_t)gy * a.px + gx;
   const int xm = gx == 0 ? nx - 1 : gx - 1, xp = gx == nx - 1 ? 0 : gx + 1;
   const int ym = gy == 0 ? ny - 1 : gy - 1, yp = gy == ny - 1 ? 0 : gy + 1;
   // Destination node and direction of population k after streaming.
@@ -590,7 +591,7 @@ __device__ __forceinline__ void collide_stream(
       dx = gx;
       dk[k] = opp_of(k);
     }
-    dst[k] = (size_t)dy * nx + dx;
+    dst[k] = (size_t)dy * a.px + dx;
   }
   constexpr bool MIX = Prec<P>::MIX;
   const T ux = m.ux, uy = m.uy, uu = m.uu, rho = m.rho;
@@ -751,7 +752,7 @@ __device__ __forceinline__ void phi_global(const KArgs<P> &a, int sx, int sy,
                                            typename Prec<P>::T *out, int plane,
                                            int idx) {
   typedef typename Prec<P>::T T;
-  const size_t q = (size_t)sy * a.nx + sx;
+  const size_t q = (size_t)sy * a.px + sx;
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     T mov[8], err;
@@ -772,14 +773,14 @@ __device__ __forceinline__ void phi_global(const KArgs<P> &a, int sx, int sy,
 // instead of two: what counts on a grid of one wave of tiles) where registers
 // are left for them. us per step in 2 / 3 / 4 CTAs (e: loaded early): N = 3,
 // 256^2 4.49e / 4.50e / 4.69e (4.87 before); N = 5, 256^2 6.23e / 7.05e /
-// 13.4e (6.43 before), 512^2 23.2e / 24.1e; N = 4, 1501 x 997 116e / 105.7e,
-// 105.9 / 101 (104 before); N = 3 unequal densities, 1024^2 74e / 65e, 60.5 /
-// 56.9 (62.4 before), 400 x 200 8.2e / 7.0e, 6.9 / 7.1 (7.1 before); Eq. N40,
-// N = 4, 512^2 18.3e / 17.1e, 17.3 / 18.0 (17.2 before).
+// 13.4e (6.43 before), 512^2 23.2e / 24.1e; N = 4, 301 x 203 - / 5.61e / 6.41
+// (7.18 before); unequal densities: N = 3, 1024^2 74e / 65e, 60.5 / 56.9 (62.4
+// before), 400 x 200 8.2e / 7.0e, 6.9 / 7.1 (7.1 before), N = 4, 701 x 503
+// - / 29.2 / 32.0 (35.0 before); Eq. N40, N = 4, 512^2 18.3e / 16.9e / 18.1.
 template <int P, int NP, bool NU, bool G40> struct TileMin {
   static constexpr bool F32 = P == LBM_FP32;
-  static constexpr bool EARLY = F32 && !NU && (NP == 2 || NP == 4);
-  static constexpr int CTAS = !F32 ? 0 : (NP == 4 ? 2 : (!G40 && (NU || NP != 2) ? 4 : 3));
+  static constexpr bool EARLY = F32 && !NU && NP != 1;
+  static constexpr int CTAS = !F32 ? 0 : (NP == 4 ? 2 : (NP == 1 || (NU && !G40 && NP == 2) ? 4 : 3));
 };
 
 template <int P, int NP, bool NU, bool WALL, bool G40>
@@ -807,7 +808,7 @@ __global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel
   T hreg[NP][9], perr[NP];
   {
     const int sx = wrap(gx, nx), sy = wrap_y<WALL>(gy, ny);
-    const size_t q = (size_t)sy * nx + sx;
+    const size_t q = (size_t)sy * a.px + sx;
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
       hreg[i][0] = ldg(a.h0_in + (size_t)i * V + q);
@@ -817,7 +818,7 @@ __global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel
           node_phi<P>(hreg[i][0], &hreg[i][1], pp, perr[i], a.sh_ld);
     }
   }
-  const size_t q = (size_t)(active ? gy : 0) * nx + (active ? gx : 0);
+  const size_t q = (size_t)(active ? gy : 0) * a.px + (active ? gx : 0);
   T g[9], up[2];
   auto load_rest = [&] {  // the node's NS populations and u(t-1)
     if (active) {
@@ -887,18 +888,19 @@ __global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel
 
   if (a.mode == MODE_MOMENTS) {
     if (!active) return;
+    const size_t qo = (size_t)gy * nx + gx, Vo = (size_t)nx * ny;  // dense fields
     if (a.o_phi)
 #pragma unroll
-      for (int i = 0; i < NP; ++i) a.o_phi[(size_t)i * V + q] = (double)m.ph[i];
+      for (int i = 0; i < NP; ++i) a.o_phi[(size_t)i * Vo + qo] = (double)m.ph[i];
     if (a.o_c)
 #pragma unroll
-      for (int k = 0; k <= NP; ++k) a.o_c[(size_t)k * V + q] = (double)m.cc[k];
+      for (int k = 0; k <= NP; ++k) a.o_c[(size_t)k * Vo + qo] = (double)m.cc[k];
     if (a.o_u) {
-      a.o_u[q] = (double)m.ux;
-      a.o_u[V + q] = (double)m.uy;
+      a.o_u[qo] = (double)m.ux;
+      a.o_u[Vo + qo] = (double)m.uy;
     }
-    if (a.o_p) a.o_p[q] = (double)m.pr;
-    if (a.o_rho) a.o_rho[q] = (double)m.rho;
+    if (a.o_p) a.o_p[qo] = (double)m.pr;
+    if (a.o_rho) a.o_rho[qo] = (double)m.rho;
     return;
   }
   if (a.mode == MODE_DIAG) {
@@ -1139,14 +1141,15 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
   const int nmine = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
 
   // FP32 tiles on the edge of a periodic grid: which wrapped halo column
-  // (1: x = -1, staged from x = nx - 4 .. nx - 1; 2: x = nx, from 0 .. 3)
-  // and row (1: y = -1 from ny - 1; 2: y = ny from 0; none with walls,
-  // whose ghost rows repeat a row of the box) are staged with the tile.
+  // (1: x = -1, in the 16 bytes of columns that hold x = nx - 1; 2: x = nx,
+  // from 0 .. 3, also where the tile overhangs the grid) and row (1: y = -1
+  // from ny - 1; 2: y = ny from 0; none with walls, whose ghost rows repeat a
+  // row of the box) are staged with the tile.
   auto halo_x = [&](int x0) {
-    return !G::WRAP ? 0 : (x0 == 0 ? 1 : (x0 + BX == nx ? 2 : 0));
+    return !G::WRAP ? 0 : (x0 == 0 ? 1 : (x0 + BX >= nx ? 2 : 0));
   };
   auto halo_y = [&](int y0) {
-    return (!G::WRAP || WALL) ? 0 : (y0 == 0 ? 1 : (y0 + TBY == ny ? 2 : 0));
+    return (!G::WRAP || WALL) ? 0 : (y0 == 0 ? 1 : (y0 + TBY >= ny ? 2 : 0));
   };
   auto issue = [&](int j) {  // thread 0: TMA loads of my j-th tile
     const int t = blockIdx.x + j * gridDim.x;
@@ -1164,7 +1167,7 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
     if constexpr (G::WRAP) {
       unsigned char *w = st + St::BASE;
       if (wx) {
-        const int xs = wx == 1 ? nx - G::HXR : 0;
+        const int xs = wx == 1 ? (nx - 1) / G::HXR * G::HXR : 0;
         tma_load_3d(w, &maps.hmx, xs, y0 - 1, 0, b);
         tma_load_3d(w + St::XHM, &maps.h0x, xs, y0 - 1, 0, b);
         tma_load_3d(w + St::XHM + St::XH0, &maps.ppx, xs, y0 - 1, 0, b);
@@ -1272,7 +1275,7 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
           const int ox = arr == 0 ? G::HXM : (arr == 3 ? G::UOX : G::HXR);
           const int oy = arr < 2 ? 1 : G::RY;
           const size_t q = (size_t)pl * a.V +
-                           (size_t)wrap(y0 - oy + by, ny) * nx + wrap(x0 - ox + bx, nx);
+                           (size_t)wrap(y0 - oy + by, ny) * a.px + wrap(x0 - ox + bx, nx);
           const void *src = arr == 0 ? (const void *)(a.hm_in + q)
                             : arr == 1 ? (const void *)(a.h0_in + q)
                             : arr == 2 ? (const void *)(a.pp_in + q)
@@ -1336,7 +1339,7 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
 #pragma unroll
         for (int i = 0; i < NP; ++i) sph[i] = spp[(i * G::HBP + r) * G::WR + c];
       } else {
-        const size_t qs = source_node<WALL>(xn, yn, k, nx, ny);
+        const size_t qs = source_node<WALL>(xn, yn, k, nx, ny, a.px);
         sux = ldg(a.u_in + qs);
         suy = ldg(a.u_in + a.V + qs);
         spr = ldg(a.u_in + 2 * a.V + qs);
@@ -1378,6 +1381,47 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
         if (err) err[i] = e;
       }
     };
+    // phi at tile position (lx, ly), at most one beyond the grid
+    auto edge_phi = [&](int lx, int ly) {
+      const int rx = x0 - 1 + lx;
+      // a wall's ghost row is the adjacent row of the box
+      const int ry = WALL ? wrap_y<WALL>(y0 - 1 + ly, ny) : y0 - 1 + ly, by = ry - y0 + 1;
+      const bool inx = rx >= 0 && rx < nx, iny = ry >= 0 && ry < ny;
+      if (PATCH || (inx && iny)) {
+        box_phi(lx - 1 + G::HXM, lx - 1 + G::HXR, by, nullptr, ly);
+        return;
+      }
+      if constexpr (G::WRAP) {
+        // the staged wrapped column or row
+        const int wx = halo_x(x0), wy = halo_y(y0);
+        const unsigned char *w = st + St::BASE;
+        auto wrap_phi = [&](const Sm *hmb, const T *h0b, const T *ppb, int pm, int pr,
+                            int om, int orr) {
+#pragma unroll
+          for (int i = 0; i < NP; ++i) {
+            T mov[8], e;
+#pragma unroll
+            for (int k = 1; k < 9; ++k) mov[k - 1] = to_T(hmb[(i * 8 + k - 1) * pm + om]);
+            sphi[i * PL + ly * SW + lx] =
+                node_phi<P>(h0b[i * pr + orr], mov, ppb[i * pr + orr], e, a.sh_ld);
+          }
+        };
+        if (iny && ((rx < 0 && wx == 1) || (rx >= nx && wx == 2))) {
+          const int c = rx < 0 ? (nx - 1) % G::HXR : 0;
+          wrap_phi((const Sm *)w, (const T *)(w + St::XHM), (const T *)(w + St::XHM + St::XH0),
+                   G::HB * G::HXM, G::HB * G::HXR, by * G::HXM + c, by * G::HXR + c);
+          return;
+        }
+        if (inx && ((ry < 0 && wy == 1) || (ry >= ny && wy == 2))) {
+          w += St::XHM + St::XH0 + St::XPP;
+          wrap_phi((const Sm *)w, (const T *)(w + St::YHM), (const T *)(w + St::YHM + St::YH0),
+                   G::WM, G::WR, lx - 1 + G::HXM, lx - 1 + G::HXR);
+          return;
+        }
+      }
+      // corners, grids one tile wide or high (and the 16-bit forms' edges)
+      phi_global<P, NP, WALL>(a, wrap(rx, nx), wrap_y<WALL>(ry, ny), sphi, PL, ly * SW + lx);
+    };
     // own node (ly = ty + 1, lx = tx + 1; box column tx + HX, row ty + 1):
     // its populations go to registers once, for phi and for the collision.
     T perr[NP], hreg[NP][9], g[9], pp[NP];
@@ -1408,9 +1452,9 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
       for (int i = 0; i < NP; ++i)
         sphi[i * PL + (ty + 1) * SW + tx + 1] =
             node_phi<P>(hreg[i][0], &hreg[i][1], pp[i], perr[i], a.sh_ld);
-    } else {
-      phi_global<P, NP, WALL>(a, wrap(gx, nx), wrap_y<WALL>(gy, ny), sphi, PL,
-                        (ty + 1) * SW + tx + 1);
+    } else if (gx <= nx && gy <= ny) {
+      // the position one beyond the grid in a tile that overhangs it
+      edge_phi(tx + 1, ty + 1);
     }
     // ring positions on warps 1..3 (threads 32 .. 32 + NRING - 1): warp 0
     // holds the thread that issues the stage refills
@@ -1419,49 +1463,7 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
     if (tid >= 32 && tid < 32 + NRING) {
       int lx, ly;
       ring_pos_1<TBY>(tid - 32, lx, ly);
-      const int rx = x0 - 1 + lx, ry = y0 - 1 + ly;
-      const bool inx = rx >= 0 && rx < nx, iny = ry >= 0 && ry < ny;
-      if (PATCH) {
-        // a wall's ghost row is the adjacent row of the box
-        const int by = WALL ? wrap_y<WALL>(ry, ny) - y0 + 1 : ly;
-        box_phi(lx - 1 + G::HXM, lx - 1 + G::HXR, by, nullptr, ly);
-      } else if (inx && iny) {
-        box_phi(lx - 1 + G::HXM, lx - 1 + G::HXR, ly, nullptr);
-      } else if constexpr (G::WRAP) {
-        // staged wrapped column or row, a wall's ghost row from the box, or
-        // (corners, ragged tails) global memory
-        const int wx = halo_x(x0), wy = halo_y(y0);
-        const unsigned char *w = st + St::BASE;
-        auto wrap_phi = [&](const Sm *hmb, const T *h0b, const T *ppb, int pm, int pr,
-                            int om, int orr) {
-#pragma unroll
-          for (int i = 0; i < NP; ++i) {
-            T mov[8], e;
-#pragma unroll
-            for (int k = 1; k < 9; ++k) mov[k - 1] = to_T(hmb[(i * 8 + k - 1) * pm + om]);
-            sphi[i * PL + ly * SW + lx] =
-                node_phi<P>(h0b[i * pr + orr], mov, ppb[i * pr + orr], e, a.sh_ld);
-          }
-        };
-        if (iny && ((rx < 0 && wx == 1) || (rx >= nx && wx == 2))) {
-          const int c = rx < 0 ? G::HXR - 1 : 0;
-          wrap_phi((const Sm *)w, (const T *)(w + St::XHM), (const T *)(w + St::XHM + St::XH0),
-                   G::HB * G::HXM, G::HB * G::HXR, ly * G::HXM + c, ly * G::HXR + c);
-        } else if (inx && WALL) {
-          box_phi(lx - 1 + G::HXM, lx - 1 + G::HXR, wrap_y<WALL>(ry, ny) - y0 + 1, nullptr,
-                  ly);
-        } else if (inx && ((ry < 0 && wy == 1) || (ry >= ny && wy == 2))) {
-          w += St::XHM + St::XH0 + St::XPP;
-          wrap_phi((const Sm *)w, (const T *)(w + St::YHM), (const T *)(w + St::YHM + St::YH0),
-                   G::WM, G::WR, lx - 1 + G::HXM, lx - 1 + G::HXR);
-        } else {
-          phi_global<P, NP, WALL>(a, wrap(rx, nx), wrap_y<WALL>(ry, ny), sphi, PL,
-                                  ly * SW + lx);
-        }
-      } else {
-        phi_global<P, NP, WALL>(a, wrap(rx, nx), wrap_y<WALL>(ry, ny), sphi, PL,
-                                ly * SW + lx);
-      }
+      if (WHOLE || (x0 - 1 + lx <= nx && y0 - 1 + ly <= ny)) edge_phi(lx, ly);
     }
     const T upx = sup[(ty + G::UOY) * G::UW + tx + G::UOX];
     const T upy = sup[(G::UH + ty + G::UOY) * G::UW + tx + G::UOX];
@@ -1520,22 +1522,24 @@ __global__ void init_phi_kernel(const KArgs<P> a, const double *c,
   typedef typename Prec<P>::T T;
   const double rt[5] = {r0, r1, r2, r3, r4};
   const double rN = rt[NP];
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < a.V;
+  const size_t Vd = (size_t)a.nx * a.ny;  // dense inputs and phid, pitched state
+  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < Vd;
        q += (size_t)gridDim.x * blockDim.x) {
-    const double cN = c[(size_t)NP * a.V + q];
+    const size_t qp = q / a.nx * a.px + q % a.nx;
+    const double cN = c[(size_t)NP * Vd + q];
     double ph[NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      const double ci = c[(size_t)i * a.V + q];
+      const double ci = c[(size_t)i * Vd + q];
       ph[i] = (2.0 * (rt[i] * ci - rN * cN) - (rt[i] - rN)) / (rt[i] + rN);
     }
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      a.pp_out[(size_t)i * a.V + q] = (T)ph[i];
-      phid[(size_t)i * a.V + q] = ph[i];
+      a.pp_out[(size_t)i * a.V + qp] = (T)ph[i];
+      phid[(size_t)i * Vd + q] = ph[i];
     }
-    a.u_out[q] = u ? (T)u[q] : T(0);
-    a.u_out[a.V + q] = u ? (T)u[a.V + q] : T(0);
+    a.u_out[qp] = u ? (T)u[q] : T(0);
+    a.u_out[a.V + qp] = u ? (T)u[Vd + q] : T(0);
   }
 }
 
@@ -1577,9 +1581,11 @@ __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
   T *h0 = a.h0_out;
   Sm *hm = a.hm_out;
   Sm *gm = a.gm_out;
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < V;
-       q += (size_t)gridDim.x * blockDim.x) {
-    const int x = (int)(q % nx), y = (int)(q / nx);
+  const size_t Vd = (size_t)nx * ny;
+  for (size_t qd = blockIdx.x * (size_t)blockDim.x + threadIdx.x; qd < Vd;
+       qd += (size_t)gridDim.x * blockDim.x) {
+    const int x = (int)(qd % nx), y = (int)(qd / nx);
+    const size_t q = (size_t)y * a.px + x;
     double ph[NP], lp[NP];
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
@@ -1589,13 +1595,13 @@ __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
 #pragma unroll
         for (int dx = -1; dx <= 1; ++dx)
           s[(dy + 1) * 3 + dx + 1] =
-              phid[(size_t)i * V + (size_t)wrap_y<WALL>(y + dy, ny) * nx + wrap(x + dx, nx)];
+              phid[(size_t)i * Vd + (size_t)wrap_y<WALL>(y + dy, ny) * nx + wrap(x + dx, nx)];
       ph[i] = s[4];
       lp[i] = laplacian<double, 3>(s, 1, 1);
     }
     double cc[NP + 1], rho, hf[NP];
     local_algebra<LBM_FP64, NP>(d, ph, cc, rho, hf);
-    const double ux = uin ? uin[q] : 0.0, uy = uin ? uin[V + q] : 0.0;
+    const double ux = uin ? uin[qd] : 0.0, uy = uin ? uin[Vd + qd] : 0.0;
     const double uu = ux * ux + uy * uy;
     if constexpr (Prec<P>::REF) a.u_out[2 * V + q] = (T)p0;
 #pragma unroll
@@ -1604,7 +1610,7 @@ __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
       const double geq =
           w_of<double>(k) * (3.0 * p0 + rho * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu));
       if constexpr (Prec<P>::MIX) {
-        const size_t qs = source_node<WALL>(x, y, k, nx, ny);
+        const size_t qs = source_node<WALL>(x, y, k, nx, ny, a.px);
         const T sux = a.u_out[qs], suy = a.u_out[V + qs];
         // every source starts at p0 (stored as its p(t-1) above)
         const T ref = Prec<P>::REF ? g_refp(cdotu(k, sux, suy), sux, suy, (T)p0,
@@ -1627,7 +1633,7 @@ __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
         const double heq =
             w_of<double>(k) * (aC + 3.0 * ph[i] * (cx_of(k) * ux + cy_of(k) * uy));
         if constexpr (Prec<P>::MIX) {
-          const size_t qs = source_node<WALL>(x, y, k, nx, ny);
+          const size_t qs = source_node<WALL>(x, y, k, nx, ny, a.px);
           const T ref = Prec<P>::REF ? adv_units(cdotu(k, a.u_out[qs], a.u_out[V + qs]),
                                                  a.pp_out[(size_t)i * V + qs], T(3) * a.sh_st)
                                      : T(0);
@@ -1667,7 +1673,10 @@ namespace lbm {
 // kernel's single CTA fetches its tensor maps and fills its stages first. us
 // per step, pipelined / generic: N = 3, 64^2 4.04 / 3.35, 256^2 5.29 / 4.45,
 // 384^2 (576 tiles) 7.88 / 7.65; N = 5, 256^2 8.40 / 6.23, 384^2 13.1 / 11.0,
-// 512^2 (1024 tiles) 20.8 / 23.2. The 16-bit forms' decode makes the generic
+// 512^2 (1024 tiles) 20.8 / 23.2. Grids that are not whole tiles, beyond that
+// line: 1501 x 997 (rows padded to 1504) N = 4 85.6 / 101, N = 2 42.0 / 54.2;
+// 1200 x 900 N = 5 141 -> 81.6 with the wrapped column and row of overhanging
+// tiles staged. The 16-bit forms' decode makes the generic
 // kernel slower at every size (BF16 N = 3, 128^2 4.9 / 6.6).
 template <int P> inline bool pipelined_pays(const Grid &g) {
   return P != LBM_FP32 || g.tma_all || (long long)tiles_x(g.nx) * tiles_y(g.ny) > 4 * 152;
@@ -1747,7 +1756,7 @@ bool encode_tma_p(const Consts &c, Grid &g, EncodeTiledFn enc) {
   if constexpr (P == LBM_FP64) {
     return false;
   } else {
-    if (!enc || g.nx % 8 != 0) return false;
+    if (!enc || g.px % 8 != 0) return false;
     const int NP = c.NP;
     auto enc3 = [&](CUtensorMap *m, void *base, size_t es, int planes, int bw,
                     int bh, int bp) {
@@ -1755,8 +1764,8 @@ bool encode_tma_p(const Consts &c, Grid &g, EncodeTiledFn enc) {
           es == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_UINT16;
       const cuuint64_t dims[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny,
                                   (cuuint64_t)planes};
-      const cuuint64_t strides[2] = {(cuuint64_t)g.nx * es,
-                                     (cuuint64_t)g.nx * g.ny * es};
+      const cuuint64_t strides[2] = {(cuuint64_t)g.px * es,
+                                     (cuuint64_t)g.px * g.ny * es};
       const cuuint32_t box[3] = {(cuuint32_t)bw, (cuuint32_t)bh, (cuuint32_t)bp};
       const cuuint32_t estr[3] = {1, 1, 1};
       return enc(m, dt, 3, base, dims, strides, box, estr,
@@ -1792,7 +1801,7 @@ cudaError_t launch_init_np(const Consts &c, const Grid &g, int cur,
   // pointers at cur ^ 1, so pass cur ^ 1.
   const KArgs<P> a = make_args<P>(c, g, cur ^ 1, MODE_STEP, Outputs{});
   const int threads = 256;
-  size_t blocks = (g.V + threads - 1) / threads;
+  size_t blocks = ((size_t)g.nx * g.ny + threads - 1) / threads;
   if (blocks > 65535u * 16u) blocks = 65535u * 16u;
   init_phi_kernel<P, NP><<<(unsigned)blocks, threads, 0, s>>>(
       a, cin, uin, g.scratch, c.rho_t[0], c.rho_t[1], c.rho_t[2], c.rho_t[3], c.rho_t[4]);
