@@ -834,9 +834,7 @@ lbm_status lbm_nphase_moments(lbm_nphase_t *h, double *phi, double *c,
       if (e != cudaSuccess) return cuda_fail(h, e);
     }
   }
-  e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  return check_err(h);
+  return check_err(h);  // synchronises
 }
 
 lbm_status lbm_nphase_diagnostics(lbm_nphase_t *h, double *mass, double *ke,

@@ -312,6 +312,25 @@ template <int P, int NP> struct Own3 {
   T h[NP][15], g[15], pp[NP], up[3];
 };
 
+// The NS populations of a node alone, as load_own3 loads them.
+template <int P, typename At>
+__device__ __forceinline__ void load_g3(const KArgs<P> &a, const At &at,
+                                        typename Prec<P>::T (&g)[15]) {
+  typedef typename Prec<P>::T T;
+  const size_t V = a.V;
+#pragma unroll
+  for (int k = 1; k < 15; ++k) {
+    g[k] = to_T(ldg(at.own(a.gm_in + (size_t)(k - 1) * V)));
+    if constexpr (Prec<P>::REF) {
+      const T ux = ldg(at.src(a.u_in, k)), uy = ldg(at.src(a.u_in + V, k)),
+              uz = ldg(at.src(a.u_in + 2 * V, k));
+      g[k] = __fadd_rn(g[k], g_ref3p(cdotu3(k, ux, uy, uz), ux, uy, uz,
+                                     ldg(at.src(a.u_in + 3 * V, k)), a.rho_base * a.sg_st,
+                                     T(3) * a.sg_st));
+    }
+  }
+}
+
 template <int P, int NP, typename At>
 __device__ __forceinline__ void load_own3(const KArgs<P> &a, const At &at, Own3<P, NP> &o) {
   typedef typename Prec<P>::T T;
@@ -537,6 +556,53 @@ __device__ __forceinline__ void collide3(
   if constexpr (Prec<P>::REF) *at.own(a.u_out + 3 * V) = pr;
 }
 
+template <int P, int NP>
+__device__ __forceinline__ void write_macros3(const KArgs<P> &a, size_t q,
+                                              const typename Prec<P>::T *ph,
+                                              const typename Prec<P>::T *cc,
+                                              const typename Prec<P>::T *u,
+                                              typename Prec<P>::T pr,
+                                              typename Prec<P>::T rho) {
+  const size_t V = a.V;
+  if (a.o_phi)
+    for (int i = 0; i < NP; ++i) a.o_phi[(size_t)i * V + q] = (double)ph[i];
+  if (a.o_c)
+    for (int k = 0; k <= NP; ++k) a.o_c[(size_t)k * V + q] = (double)cc[k];
+  if (a.o_u)
+    for (int d = 0; d < 3; ++d) a.o_u[(size_t)d * V + q] = (double)u[d];
+  if (a.o_p) a.o_p[q] = (double)pr;
+  if (a.o_rho) a.o_rho[q] = (double)rho;
+}
+
+// mass_k, ke and umax of a 32 x 4 x 2 tile: warp shuffle, then warps in fixed
+// order.
+template <int P, int NP>
+__device__ __forceinline__ void diag_partials3(const KArgs<P> &a, bool active,
+                                               const typename Prec<P>::T *cc,
+                                               typename Prec<P>::T rho,
+                                               typename Prec<P>::T uu,
+                                               double (*sred)[8]) {
+  const int tid = (threadIdx.z * BY3 + threadIdx.y) * BX3 + threadIdx.x;
+  const int lane = tid & 31, wid = tid >> 5;
+#pragma unroll
+  for (int k = 0; k <= NP + 2; ++k) {
+    double v;
+    if (k <= NP) v = active ? (double)cc[k] : 0.0;
+    else if (k == NP + 1) v = active ? 0.5 * (double)rho * (double)uu : 0.0;
+    else v = active ? sqrt((double)uu) : 0.0;
+    v = (k == NP + 2) ? warp_max(v) : warp_sum(v);
+    if (lane == 0) sred[wid][k] = v;
+  }
+  __syncthreads();
+  if (tid <= NP + 2) {
+    double v = sred[0][tid];
+    for (int w = 1; w < NT3 / 32; ++w)
+      v = (tid == NP + 2) ? fmax(v, sred[w][tid]) : v + sred[w][tid];
+    const size_t b = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    a.red[b * (NP + 3) + tid] = v;
+  }
+}
+
 template <int P, int NP, bool NU, bool WALL>
 __global__ void __launch_bounds__(NT3, P == LBM_FP64 ? 1 : 2)
     tile3_kernel(const KArgs3<P> A) {
@@ -652,36 +718,11 @@ __global__ void __launch_bounds__(NT3, P == LBM_FP64 ? 1 : 2)
   T F[3], u[3], uu, pr;
   macros3<P, NP>(a, gp, Cv, rho, gr, own.g, u, F, uu, pr);
   if (a.mode == MODE_MOMENTS) {
-    if (!active) return;
-    if (a.o_phi)
-      for (int i = 0; i < NP; ++i) a.o_phi[(size_t)i * V + q] = (double)ph[i];
-    if (a.o_c)
-      for (int k = 0; k <= NP; ++k) a.o_c[(size_t)k * V + q] = (double)cc[k];
-    if (a.o_u)
-      for (int d = 0; d < 3; ++d) a.o_u[(size_t)d * V + q] = (double)u[d];
-    if (a.o_p) a.o_p[q] = (double)pr;
-    if (a.o_rho) a.o_rho[q] = (double)rho;
+    if (active) write_macros3<P, NP>(a, q, ph, cc, u, pr, rho);
     return;
   }
   if (a.mode == MODE_DIAG) {
-    const int lane = tid & 31, wid = tid >> 5;
-#pragma unroll
-    for (int k = 0; k <= NP + 2; ++k) {
-      double v;
-      if (k <= NP) v = active ? (double)cc[k] : 0.0;
-      else if (k == NP + 1) v = active ? 0.5 * (double)rho * (double)uu : 0.0;
-      else v = active ? sqrt((double)uu) : 0.0;
-      v = (k == NP + 2) ? warp_max(v) : warp_sum(v);
-      if (lane == 0) sred[wid][k] = v;
-    }
-    __syncthreads();
-    if (tid <= NP + 2) {
-      double v = sred[0][tid];
-      for (int w = 1; w < NT3 / 32; ++w)
-        v = (tid == NP + 2) ? fmax(v, sred[w][tid]) : v + sred[w][tid];
-      const size_t b = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-      a.red[b * (NP + 3) + tid] = v;
-    }
+    diag_partials3<P, NP>(a, active, cc, rho, uu, sred);
     return;
   }
   if (!active) return;
@@ -780,6 +821,52 @@ __global__ void __launch_bounds__(NT3) pot3_kernel(const KArgs3<P> A) {
       *at.own(A.C + (size_t)i * a.V) = Ci;
     }
   });
+}
+
+// Fields (MODE_MOMENTS) or per-CTA partial sums of the diagnostics (MODE_DIAG)
+// from phi(t) in memory: the stencils and the NS populations are all a node
+// needs (C_i is local), so h is read once, by phi3_kernel. us per call
+// before (tile kernel, phi on 3.2 or 6.8 positions per node) -> now: FP32 256^3
+// N = 3 1390 -> 939, BF16 128^3 with walls 350 -> 216, FP64 96^3 648 -> 499, FP32
+// 96^3 unequal densities 189 -> 110.
+template <int P, int NP, bool NU, bool WALL>
+__global__ void __launch_bounds__(NT3) macro3_kernel(const KArgs3<P> A) {
+  typedef typename Prec<P>::T T;
+  const KArgs<P> &a = A.a;
+  const int nx = a.nx, ny = a.ny, nz = A.nz;
+  __shared__ double sred[NT3 / 32][8];
+  T ph[NP], cc[NP + 1], rho = T(0), u[3], uu = T(0), pr = T(0);
+  size_t q = 0;
+  bool active = false;
+  for_node3<WALL>(nx, ny, nz, [&](const auto &at) {
+    active = true;
+    q = at.own(a.pp_out) - a.pp_out;
+    T gp[NP][3], Cv[NP], lp[NP], hf[NP], g[15], gr[3] = {T(0), T(0), T(0)}, F[3];
+    load_g3<P>(a, at, g);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const T *z = a.pp_out + (size_t)i * a.V;
+      ph[i] = *at.own(z);
+      stencil3m(z, at, ph[i], gp[i], lp[i]);
+    }
+    local_algebra<P, NP, !NU>(a, ph, cc, rho, hf);
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      T Ci = a.bulk * hf[i];
+#pragma unroll
+      for (int j = 0; j < NP; ++j) Ci -= a.lam[i][j] * lp[j];
+      Cv[i] = Ci;
+      if constexpr (NU)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) gr[d] += a.kap[i] * gp[i][d];
+    }
+    macros3<P, NP>(a, gp, Cv, rho, gr, g, u, F, uu, pr);
+  });
+  if (a.mode == MODE_MOMENTS) {
+    if (active) write_macros3<P, NP>(a, q, ph, cc, u, pr, rho);
+  } else {
+    diag_partials3<P, NP>(a, active, cc, rho, uu, sred);
+  }
 }
 
 template <int P, int NP, bool NU, bool WALL>
@@ -1267,6 +1354,14 @@ cudaError_t launch_tile3_t(const Consts &c, const Grid &g, int cur, int mode,
   A.nz = g.nz;
   A.C = (T *)g.scratch;
   const dim3 tiles(tiles3_x(g.nx), tiles3_y(g.ny), tiles3_z(g.nz)), tblock(BX3, BY3, BZ3);
+  if (mode != MODE_STEP && g.split3) {
+    // phi(t) goes to the buffer the next step writes
+    phi3_kernel<P, NP, WALL><<<tiles, tblock, 0, s>>>(A);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    macro3_kernel<P, NP, NU, WALL><<<tiles, tblock, 0, s>>>(A);
+    return cudaGetLastError();
+  }
   if (mode == MODE_STEP && g.split3) {
     if constexpr (P == LBM_FP32 && NP <= 3 && !NU) {
       if (march3_pays(g, NP)) {
