@@ -1083,7 +1083,12 @@ template <int P, int NP> struct TmaStage {
   static constexpr uint32_t YTX =
       (uint32_t)((size_t)8 * NP * G::WM * sizeof(Sm) + (size_t)2 * NP * G::WR * sizeof(T));
   static constexpr size_t SPHI = al((size_t)NP * (G::TBY + 2) * (BX + 2) * sizeof(T));
-  static constexpr int S = G::S;
+  // Stages. FP32, N = 3: three of 49 KB and one CTA per SM; two and two CTAs
+  // hold 216 KB, which leaves L1 too little for the stores. us per step, 2
+  // stages x 2 CTAs / 2 x 1 / 3 x 1 / 4 x 1: 2048^2 213 / 184 / 165 / 215,
+  // 1504 x 1000 69.1 / 68.2 / 60.3 / 67.1, 1024^2 48.8 / 49.0 / 45.3 / 46.2.
+  static constexpr int S = G::WIDE && NP == 2 ? 3 : G::S;
+  static constexpr int CTAS = G::WIDE && NP == 2 ? 1 : 8;  // most per SM
   // FP32: two phi tiles (one barrier per tile, below); 16-bit forms: one
   static constexpr int NPHI = G::WIDE ? 2 : 1;
   static constexpr size_t SMEM = S * BYTES + NPHI * SPHI + 64;
@@ -1706,6 +1711,7 @@ cudaError_t launch_tile_t(const Consts &c, const Grid &g, int cur, int mode,
         if (e != cudaSuccess) return e;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        per_sm = per_sm > St::CTAS ? St::CTAS : per_sm;
         mc = (per_sm > 0 ? per_sm : 1) * sms;
       }
       const int ntx = tiles_x(g.nx), ntiles = ntx * ((g.ny + TBY - 1) / TBY);
