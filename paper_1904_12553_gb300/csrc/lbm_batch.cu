@@ -602,10 +602,19 @@ lbm_status build_schedule(lbm_nphase_batch_t *b, lbm_nphase_batch_schedule s) {
   std::vector<double> icost;
   for (int c : order) {
     const size_t nt = tiles_for(b->cases[c]->prm, tby);
-    for (size_t t = 0; t < nt; ++t) {
-      items.push_back(make_int2(c, (int)t));
-      icost.push_back(b->cases[c]->prm.N);
+    // Dynamic chunks: the items of a chunk lie G tiles apart, G the chunks in
+    // flight (or in the case), so that the CTAs, each on the k-th item of its
+    // chunk, read neighbouring tiles at a time. us per step, consecutive
+    // tiles / G apart, chunks of 4: one 2048^2 N = 5 case 333 / 295, the 48
+    // cases of sides 64..512 370 / 353.
+    const size_t ch = s.schedule == lbm::SCHED_DYNAMIC ? (size_t)s.chunk : 1;
+    const size_t win = std::min(nt, ch * (size_t)s.ctas) / ch * ch;
+    for (size_t t0 = 0; t0 < nt; t0 += win ? win : nt) {
+      const size_t w = win ? std::min(win, nt - t0) : nt, G = w / ch;
+      for (size_t p = 0; p < w; ++p)
+        items.push_back(make_int2(c, (int)(t0 + (p < G * ch ? p % ch * G + p / ch : p))));
     }
+    icost.resize(items.size(), b->cases[c]->prm.N);
   }
   if (items.size() > b->items_cap) return LBM_ENOMEM;
   // Per-CTA lists: the cost-ordered item sequence cut into contiguous runs of
