@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(BG::NTH, 1)
                      const TmaItem *__restrict__ items, int nitems,
                      const int *__restrict__ list_off,
                      const int *__restrict__ list, int sched, int chunk,
-                     int *counter, int cur) {
+                     int *counter, int cur, int rev) {
   constexpr int S = BSt::S;
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t *bar = (uint64_t *)(smem + S * kStageStride + 2 * BSt::SPHI);
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(BG::NTH, 1)
     const int slot = j % S;
     const TmaItem d = d_next;
     if (d.c >= 0) {
-      d_next = i_after < nitems ? items[i_after] : none;
+      d_next = i_after < nitems ? items[rev ? nitems - 1 - i_after : i_after] : none;
       i_after = i_after < nitems ? next_index() : nitems;
     }
     s_slot[slot] = d;
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(BG::NTH, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     const int i0 = next_index();
     if (i0 < nitems) {
-      d_next = items[i0];
+      d_next = items[rev ? nitems - 1 - i0 : i0];
       i_after = next_index();
     }
     for (int j = 0; j < S; ++j) issue(j);
@@ -514,6 +514,7 @@ struct lbm_nphase_batch_t {
   int *d_list_off, *d_list, *d_counter;
   size_t items_cap, lists_cap;
   int nitems;
+  bool big;                // the state is beyond L2 (see walk_back)
   lbm_nphase_batch_schedule sched;
   int max_ctas[2];         // resident CTAs per tile height (generic kernel)
   int max_ctas_tma;        // resident CTAs of the pipelined kernel
@@ -556,7 +557,8 @@ cudaError_t launch_once(lbm_nphase_batch_t *b, cudaStream_t s, int cur) {
   if (b->sched.pipelined)
     lbm::batch_kernel_tma<<<grid, dim3(lbm::BX, lbm::BG::TBY), lbm::kBatchSmem, s>>>(
         b->d_cases, b->d_maps, b->n, b->d_titems, b->nitems, b->d_list_off,
-        b->d_list, b->sched.schedule, b->sched.chunk, b->d_counter, cur);
+        b->d_list, b->sched.schedule, b->sched.chunk, b->d_counter, cur,
+        cur && b->big);
   else if (ti == 0)
     lbm::batch_kernel<LBM_FP32, 4><<<grid, dim3(lbm::BX, 4), 0, s>>>(
         b->d_cases, b->d_items, b->nitems, b->d_list_off, b->d_list,
@@ -789,7 +791,12 @@ lbm_status lbm_nphase_batch_create(const lbm_nphase_params *params, int ncases,
   // Pipelined kernel: every case must have tensor maps (FP32 maps of both
   // buffers, copied next to the descriptors).
   b->tma_ok = true;
-  for (lbm_nphase_t *h : b->cases) b->tma_ok = b->tma_ok && h->g.use_tma;
+  size_t values = 0;
+  for (lbm_nphase_t *h : b->cases) {
+    b->tma_ok = b->tma_ok && h->g.use_tma;
+    values += h->g.V * (size_t)(10 * h->prm.N);
+  }
+  b->big = 4 * values >= ((size_t)48 << 20);
   b->max_ctas_tma = 0;
   if (b->tma_ok) {
     std::vector<lbm::TmaMaps> maps(2 * (size_t)ncases);

@@ -54,6 +54,7 @@ constexpr int MX3 = 32, MY3 = 8, MT3 = MX3 * MY3;
 template <int P> struct KArgs3 {
   KArgs<P> a;  // pointers, constants (u_in, u_out hold 3 planes)
   int nz;
+  bool rev3;  // step3_kernel walks the tiles from the last to the first
   typename Prec<P>::T *C;  // C_i of the split step with unequal densities
 };
 
@@ -736,9 +737,12 @@ __global__ void __launch_bounds__(NT3, P == LBM_FP64 ? 1 : 2)
 // every node to the next step's phi(t-1) array (phi3_kernel), C_i from its
 // stencils (pot3_kernel, unequal densities), then the step of every node from
 // the stencils of both in memory (step3_kernel). No barriers, and nothing is
-// computed twice: a tile with its halo sums phi on 3.2 positions per node (6.8
-// with unequal densities), a column marched in z on 1.33 and two more planes
-// per slab, and in the 16-bit forms, which are bound by instruction issue, a
+// computed twice; step3_kernel walks large boxes from the end, so that it
+// starts with what phi3_kernel read last and the next phi3_kernel with what it
+// wrote last (walk_back; FP16 96^3 N = 5 215 -> 204, FP32 101 x 93 x 87 91 ->
+// 87). A tile with its halo sums phi on 3.2 positions per node (6.8 with
+// unequal densities), a column marched in z on 1.33 and two more planes per
+// slab, and in the 16-bit forms, which are bound by instruction issue, a
 // position costs the decode of 14 slots from their sources. It costs one more
 // read of h; the stencils' reads are L1 and L2 hits.
 // us per step before (a z-marching kernel with the column's decoded values in
@@ -774,9 +778,10 @@ __device__ __forceinline__ void stencil3m(const T *z, const At &at, T c, T *g, T
 // Calls f(at) for the node of this thread, `at` an Off3 away from the walls.
 // Tiles of 32 x 4 x 2 nodes.
 template <bool WALL, typename F>
-__device__ __forceinline__ void for_node3(int nx, int ny, int nz, F f) {
-  const int x = blockIdx.x * BX3 + threadIdx.x, y = blockIdx.y * BY3 + threadIdx.y,
-            z = blockIdx.z * BZ3 + threadIdx.z;
+__device__ __forceinline__ void for_node3(int nx, int ny, int nz, F f, bool rev = false) {
+  const int x = (rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * BX3 + threadIdx.x,
+            y = (rev ? gridDim.y - 1 - blockIdx.y : blockIdx.y) * BY3 + threadIdx.y,
+            z = (rev ? gridDim.z - 1 - blockIdx.z : blockIdx.z) * BZ3 + threadIdx.z;
   if (x >= nx || y >= ny || z >= nz) return;
   if (!WALL || (y > 0 && y < ny - 1)) {
     Off3 o;
@@ -910,7 +915,7 @@ __global__ void __launch_bounds__(NT3, P == LBM_FP64 ? 1 : 2) step3_kernel(const
     T F[3], u[3], uu, pr;
     macros3<P, NP>(a, gp, Cv, rho, gr, own.g, u, F, uu, pr);
     collide3<P, NP, NU>(a, at, ph, Cv, rho, gr, J, own, u, F, uu, pr, false);
-  });
+  }, A.rev3);
 }
 
 // Eq. N31 on D3Q15 from three planes (z - 1, z, z + 1) of stride W, pairs of
@@ -1353,6 +1358,7 @@ cudaError_t launch_tile3_t(const Consts &c, const Grid &g, int cur, int mode,
   A.a = make_args<P>(c, g, cur, mode, o);
   A.nz = g.nz;
   A.C = (T *)g.scratch;
+  A.rev3 = walk_back<P>(c, g);
   const dim3 tiles(tiles3_x(g.nx), tiles3_y(g.ny), tiles3_z(g.nz)), tblock(BX3, BY3, BZ3);
   if (mode != MODE_STEP && g.split3) {
     // phi(t) goes to the buffer the next step writes

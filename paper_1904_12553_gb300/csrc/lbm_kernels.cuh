@@ -120,6 +120,7 @@ template <int P> struct alignas(16) KArgs {  // 16: bulk-copy granule
   typedef typename Prec<P>::T T;
   typedef typename Prec<P>::Sm Sm;
   int nx, ny, px;  // px: row pitch of the state's planes (nodes)
+  int rev;         // walk the tiles from the last to the first
   size_t V;        // plane stride, px ny
   const T *h0_in;
   const Sm *hm_in, *gm_in;
@@ -137,6 +138,20 @@ template <int P> struct alignas(16) KArgs {  // 16: bulk-copy granule
   T sh_ld, sh_st, sg_ld, sg_st;  // 16-bit storage: value = S * w_k * ld
 };
 
+// Whether steps from buffer 1 walk the tiles from the last to the first: they
+// start with what the step before wrote last, still in L2 (129 MB). For states
+// of 48 MB on (smaller ones stay in L2 anyway, and the order cost up to 4%). us
+// per step, same order / alternating: FP32 701 x 503 N = 5 unequal densities
+// 40.4 / 36.8, 1024^2 N = 3 unequal densities 56.8 / 55.0, 1501 x 997 N = 4 86.0
+// / 84.5, N = 2 42.1 / 40.2, 2048^2 N = 5 268.6 / 266.5; BF16 1024^2 N = 5 85.9
+// / 84.0; 48-case ensemble 357 / 350.
+template <int P> inline bool walk_back(const Consts &c, const Grid &g) {
+  const int D = g.lattice == 1 ? 3 : 2, Q = g.lattice == 1 ? 14 : 8;
+  const size_t node = (size_t)(c.NP + 1) * Q * sizeof(typename Prec<P>::Sm) +
+                      (size_t)(2 * c.NP + D) * sizeof(typename Prec<P>::T);
+  return g.V * node >= ((size_t)48 << 20);
+}
+
 template <int P>
 KArgs<P> make_args(const Consts &c, const Grid &g, int cur, int mode,
                    const Outputs &o) {
@@ -146,6 +161,7 @@ KArgs<P> make_args(const Consts &c, const Grid &g, int cur, int mode,
   a.nx = g.nx;
   a.ny = g.ny;
   a.px = g.px;
+  a.rev = mode == MODE_STEP && cur && walk_back<P>(c, g);
   a.V = g.V;
   a.h0_in = (const T *)g.h0[cur];
   a.hm_in = (const Sm *)g.hm[cur];
@@ -797,7 +813,8 @@ __global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel
   __shared__ T sC[NP][CH * CW];
 
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
-  const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY;
+  const int x0 = (a.rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * BX;
+  const int y0 = (a.rev ? gridDim.y - 1 - blockIdx.y : blockIdx.y) * BY;
   const int nx = a.nx, ny = a.ny;
   const size_t V = a.V;
   const int gx = x0 + tx, gy = y0 + ty;
@@ -1144,6 +1161,10 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * BX + tx;
   const int nx = a.nx, ny = a.ny;
   const int nmine = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+  auto tile_of = [&](int j) {  // my j-th tile
+    const int t = blockIdx.x + j * gridDim.x;
+    return a.rev ? ntiles - 1 - t : t;
+  };
 
   // FP32 tiles on the edge of a periodic grid: which wrapped halo column
   // (1: x = -1, in the 16 bytes of columns that hold x = nx - 1; 2: x = nx,
@@ -1157,7 +1178,7 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
     return (!G::WRAP || WALL) ? 0 : (y0 == 0 ? 1 : (y0 + TBY >= ny ? 2 : 0));
   };
   auto issue = [&](int j) {  // thread 0: TMA loads of my j-th tile
-    const int t = blockIdx.x + j * gridDim.x;
+    const int t = tile_of(j);
     const int x0 = (t % ntx) * BX, y0 = (t / ntx) * TBY;
     unsigned char *st = smem + (j % S) * St::BYTES;
     uint64_t *b = bar + (j % S);
@@ -1197,7 +1218,7 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
   int issued = nmine < S ? nmine : S;
   int failed_at = -1;
   for (int j = 0; j < nmine; ++j) {
-    const int t = blockIdx.x + j * gridDim.x;
+    const int t = tile_of(j);
     const int x0 = (t % ntx) * BX, y0 = (t / ntx) * TBY;
     T *sphi = (T *)(smem + S * St::BYTES + (ONEB ? (j & 1) * St::SPHI : 0));
     unsigned char *stw = smem + (j % S) * St::BYTES;
