@@ -82,8 +82,9 @@ inline K64 make_k64(const Consts &c, const Grid &g, int cur) {
   ka.ppo = (double *)g.phi_prev[cur ^ 1];
   ka.uo = (double *)g.u_prev[cur ^ 1];
   ka.C = g.scratch;
-  // the axes' factors are exactly 4 times the diagonals', and the rest slot's
-  // -20 times, so that the collision's sums close to rounding
+  // The axes' factors are exactly 4 times the diagonals', and the rest slot's
+  // -20 times, each rounded once, so that the collision's sums close as far as
+  // rounding lets them.
   const double w5 = 1.0 / 36.0, w1 = 4.0 * w5;
   Cst64 &a = ka.c;
   a.one = 1.0;
@@ -121,10 +122,10 @@ inline K64 make_k64(const Consts &c, const Grid &g, int cur) {
     a.kap[i] = c.kap[i];
     a.kapg[i] = c.kap[i] * a.gsc;
     a.kmobg[i] = c.kmob[i] * a.gsc;
-    a.kD[i] = c.tau_inv[i] * c.a[i] * w5;
+    a.kD[i] = c.tau_inv[i] * c.a[i] / 36.0;
     a.kA[i] = 4.0 * a.kD[i];
-    a.c1[i] = 3.0 * (c.tau_inv[i] + c.src[i]) * w1;
-    a.c2[i] = 3.0 * c.src[i] * w1;
+    a.c1[i] = (c.tau_inv[i] + c.src[i]) / 3.0;
+    a.c2[i] = c.src[i] / 3.0;
     a.keep[i] = 1.0 - c.tau_inv[i];
     a.ti[i] = c.tau_inv[i];
     a.kR[i] = -20.0 * a.kD[i];
@@ -137,15 +138,15 @@ inline K64 make_k64(const Consts &c, const Grid &g, int cur) {
   a.ruu = -2.7 * tg;
   a.f3 = 3.0 * ff;
   a.jh = 0.5 * c.jfac;
-  a.B1d = 3.0 * tg * w5;
+  a.B1d = tg / 12.0;
   a.B1a = 4.0 * a.B1d;
-  a.B2d = 4.5 * tg * w5;
+  a.B2d = tg / 8.0;
   a.B2a = 4.0 * a.B2d;
-  a.C1d = 3.0 * ff * w5;
+  a.C1d = ff / 12.0;
   a.C1a = 4.0 * a.C1d;
-  a.D1a = 9.0 * ff * w1;
-  a.E1a = 3.0 * ff * w1;
-  a.E2a = 4.5 * ff * c.jfac * w1;
+  a.D1a = ff;
+  a.E1a = ff / 3.0;
+  a.E2a = 0.5 * ff * c.jfac;
   return ka;
 }
 
@@ -560,9 +561,9 @@ cudaError_t launch_step64(const Consts &c, const Grid &g, int cur, cudaStream_t 
   if (!NU) {  // rho is constant: into the coefficients
     const double r = c.rho_base;
     a.c.ruu *= r;
-    a.c.B1d *= r;
+    a.c.B1d = r * c.tg_inv / 12.0;
     a.c.B1a = 4.0 * a.c.B1d;
-    a.c.B2d *= r;
+    a.c.B2d = r * c.tg_inv / 8.0;
     a.c.B2a = 4.0 * a.c.B2d;
   }
   return g.grad_scheme == 1 ? launch_step64_t<NP, NU, WALL, true>(a, s)
