@@ -162,9 +162,18 @@ __device__ __forceinline__ double mul64(const Cst64 &k, double x, double y) {
   return fma(x, y, k.zero);
 }
 
-__device__ __forceinline__ void stage_cst64(Cst64 &k, const Cst64 &c, int tid, int nt) {
-  for (int i = tid; i < (int)(sizeof(Cst64) / sizeof(double)); i += nt)
-    ((double *)&k)[i] = ((const double *)&c)[i];
+// The constants to shared memory, all of a thread's reads first (one-warp
+// blocks, 150^2 unequal densities: 19.0 -> 18.1 us per step against a loop).
+template <int NTH>
+__device__ __forceinline__ void stage_cst64(Cst64 &k, const Cst64 &c, int tid) {
+  constexpr int N = (int)(sizeof(Cst64) / sizeof(double)), M = (N + NTH - 1) / NTH;
+  double v[M];
+#pragma unroll
+  for (int m = 0; m < M; ++m)
+    if (tid + m * NTH < N) v[m] = ((const double *)&c)[tid + m * NTH];
+#pragma unroll
+  for (int m = 0; m < M; ++m)
+    if (tid + m * NTH < N) ((double *)&k)[tid + m * NTH] = v[m];
 }
 // Sums of Eq. N31 over the eight neighbours, in units of w = 1/36: the
 // gradient over 12 (or 6 g1 - g2 over 48, Eq. N40) and the Laplacian over 6.
@@ -364,10 +373,10 @@ __global__ void __launch_bounds__(TX *TY, 512 / (TX * TY))
   __shared__ double s[NP][SW * (TY + 2)];
   __shared__ Cst64 k;
   const int tid = threadIdx.x;
-  stage_cst64(k, a.c, tid, TX * TY);
-  __syncthreads();
   const int x0 = (int)(blockIdx.x % ntx) * TX, y0 = (int)(blockIdx.x / ntx) * TY;
   double ph[NP];
+  stage_cst64<TX * TY>(k, a.c, tid);
+  __syncthreads();
   tile_phi64<NP, WALL, TX, TY>(a, k, x0, y0, tid, s, ph);
   __syncthreads();
   const int x = x0 + tid % TX, y = y0 + tid / TX;
@@ -424,10 +433,10 @@ __global__ void __launch_bounds__(TX *TY) pot64_kernel(const __grid_constant__ K
   __shared__ double s[NP][SW * (TY + 2)];
   __shared__ Cst64 k;
   const int tid = threadIdx.x;
-  stage_cst64(k, a.c, tid, TX * TY);
-  __syncthreads();
   const int x0 = (int)(blockIdx.x % ntx) * TX, y0 = (int)(blockIdx.x / ntx) * TY;
   double ph[NP];
+  stage_cst64<TX * TY>(k, a.c, tid);
+  __syncthreads();
   tile_phi64<NP, WALL, TX, TY>(a, k, x0, y0, tid, s, ph);
   __syncthreads();
   const int x = x0 + tid % TX, y = y0 + tid / TX;
@@ -460,12 +469,12 @@ __global__ void __launch_bounds__(TX *TY) pot64_kernel(const __grid_constant__ K
 
 // The collision of every node from the stencils of phi and C_i in memory
 // (9 or, Eq. N40, 17 points; L1 and L2 hits).
-template <int NP, bool NU, bool WALL, bool G40>
-__global__ void __launch_bounds__(128, 4) coll64_kernel(const __grid_constant__ K64 a) {
+template <int NP, bool NU, bool WALL, bool G40, int NTH>
+__global__ void __launch_bounds__(NTH, 512 / NTH > 32 ? 32 : 512 / NTH) coll64_kernel(const __grid_constant__ K64 a) {
   __shared__ Cst64 k;
-  stage_cst64(k, a.c, threadIdx.x, blockDim.x);
+  stage_cst64<NTH>(k, a.c, threadIdx.x);
   __syncthreads();
-  const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const size_t q = (size_t)blockIdx.x * NTH + threadIdx.x;
   const size_t V = a.V;
   if (q >= V) return;
   const int nx = a.nx, ny = a.ny;
@@ -549,8 +558,10 @@ cudaError_t launch_step64_t(const K64 &a, cudaStream_t s) {
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // one-warp blocks spread a small grid evenly; large ones take 128 threads
-    const int nt = a.V <= (size_t)152 * 32 * 32 ? 32 : 128;
-    coll64_kernel<NP, NU, WALL, G40><<<(unsigned)((a.V + nt - 1) / nt), nt, 0, s>>>(a);
+    if (a.V <= (size_t)152 * 32 * 32)
+      coll64_kernel<NP, NU, WALL, G40, 32><<<(unsigned)((a.V + 31) / 32), 32, 0, s>>>(a);
+    else
+      coll64_kernel<NP, NU, WALL, G40, 128><<<(unsigned)((a.V + 127) / 128), 128, 0, s>>>(a);
   }
   return cudaGetLastError();
 }
