@@ -793,8 +793,11 @@ __device__ __forceinline__ void for_node3(int nx, int ny, int nz, F f, bool rev 
   }
 }
 
+// Bound by the latency of its loads (51% issue active at 64 registers): five
+// CTAs per SM, us per step with 4 / 5 / 6 / 8: BF16 128^3 with walls 248 / 241 /
+// 262 / 262, FP16 96^3 N = 5 200 / 191 / 192 / 203.
 template <int P, int NP, bool WALL>
-__global__ void __launch_bounds__(NT3) phi3_kernel(const KArgs3<P> A) {
+__global__ void __launch_bounds__(NT3, P == LBM_FP64 ? 0 : 5) phi3_kernel(const KArgs3<P> A) {
   typedef typename Prec<P>::T T;
   const KArgs<P> &a = A.a;
   for_node3<WALL>(a.nx, a.ny, A.nz, [&](const auto &at) {
