@@ -964,8 +964,10 @@ __global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel
 // planes with a halo of one row and HX columns (HX * element size = 16 B,
 // the TMA alignment), completion counted on one mbarrier per stage. While a
 // tile is computed, the loads of the following S - 1 tiles are in flight.
-// Halo positions that wrap around the domain (periodic edges, wall ghost
-// rows, ragged tails) are summed from global memory instead.
+// Halo positions that wrap around the domain come from staged boxes of the
+// wrapped column and row (FP32), the patched boxes (16-bit, whole tiles) or
+// global memory (corners, other 16-bit grids); a wall's ghost row is the
+// adjacent row of the box.
 // ---------------------------------------------------------------------------
 // Pipeline shape, chosen by timing the N=5 2048^2 step on GB300: 2 stages,
 // u(t-1) staged with the tile. FP32: two phi tiles and one barrier per tile
