@@ -531,6 +531,7 @@ lbm_status lbm::create(const lbm_nphase_params *p, void *ws, size_t bytes, void 
   g.split3 = tma_allowed() && p->lattice == 1 &&
              (size_t)p->nx * p->ny * sT < ((size_t)1 << 32);
   g.march3 = g.split3 && !h->nonunif;
+  g.ring_warps = tma_allowed();
   const char *kv = getenv("LBM_NPHASE_KERNEL");
   g.tma_all = kv && strcmp(kv, "pipelined") == 0;
   g.tma3 = g.march3 && h->prec == LBM_FP32 &&

@@ -79,6 +79,7 @@ struct Grid {
   bool split3;      // D3Q15 step by the split or z-marching kernels
   bool march3;      // ... with equal densities
   bool tma3;        // ... FP32 z-marching kernel prepared (tma[] holds 4-D maps)
+  bool ring_warps;  // halo-ring warps on grids of one wave (not "generic")
   bool tma_all;     // TMA kernels at every size (LBM_NPHASE_KERNEL=pipelined)
   TmaMaps tma[2];   // its descriptors, input buffer 0 or 1
 };

@@ -799,9 +799,22 @@ template <int P, int NP, bool NU, bool G40> struct TileMin {
   static constexpr int CTAS = !F32 ? 0 : (NP == 4 ? 2 : (NP == 1 || (NU && !G40 && NP == 2) ? 4 : 3));
 };
 
-template <int P, int NP, bool NU, bool WALL, bool G40>
-__global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel(const KArgs<P> a) {
-  constexpr bool EARLY = TileMin<P, NP, NU, G40>::EARLY;
+// RW > 0 (FP32 step): that many more warps sum phi on the halo ring, one
+// position a lane, while the tile's warps load all of their nodes' values, and
+// share the positions of C_i (unequal densities). A grid of one wave is bound
+// by its chain of memory latencies, not by bandwidth (lens_256: 11 % of it):
+// the ring's is then off the chain, for ring_ctas CTAs per SM at the registers
+// that this takes. us per step, with / without: N = 3, 64^2 3.08 / 3.29, 256^2
+// 4.15 / 4.50; N = 5, 128^2 3.97 / 4.51; unequal densities: N = 3 with walls,
+// 150^2 3.79 / 4.45, 256^2 5.07 / 5.73; N = 5 with walls, 150^2 5.23 / 5.71.
+// Beyond one wave the occupancy it gives up costs more: unequal N = 2, 400 x
+// 200 (325 tiles), 7.96 with 4 warps in 3 CTAs / 6.99.
+constexpr int ring_ctas(int NP, bool NU) { return NP <= (NU ? 2 : 3) ? 2 : 1; }
+template <int P, int NP, bool NU, bool WALL, bool G40, int RW = 0>
+__global__ void __launch_bounds__(NT + 32 * RW,
+                                  RW ? ring_ctas(NP, NU) : TileMin<P, NP, NU, G40>::CTAS)
+    tile_kernel(const KArgs<P> a) {
+  constexpr bool EARLY = TileMin<P, NP, NU, G40>::EARLY || RW;
   typedef typename Prec<P>::T T;
   constexpr int RG = G40 ? 2 : 1;          // reach of a gradient stencil
   constexpr int RC = NU ? RG : 0;          // C ring radius (for grad C)
@@ -820,10 +833,19 @@ __global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel
   const int gx = x0 + tx, gy = y0 + ty;
   const bool active = gx < nx && gy < ny;
 
+  constexpr int NRING = SW * SH - BX * BY;
+  static_assert(!RW || NRING <= 32 * RW, "a ring position per lane");
+  const bool ring_warp = RW && ty >= BY;
+  if (ring_warp && tid - NT < NRING) {
+    int lx, ly;
+    ring_pos<R>(tid - NT, lx, ly);
+    phi_global<P, NP, WALL>(a, wrap(x0 - R + lx, nx), wrap_y<WALL>(y0 - R + ly, ny),
+                            &sphi[0][0], SH * SW, ly * SW + lx);
+  }
   // 1. Own node: load all h^i_k, phi_i = sum_k h^i_k (Eq. N28). hreg[i][0]
   //    holds h_0 (FP64) or d_0 (other forms); perr the rounding error of phi.
   T hreg[NP][9], perr[NP];
-  {
+  if (!ring_warp) {
     const int sx = wrap(gx, nx), sy = wrap_y<WALL>(gy, ny);
     const size_t q = (size_t)sy * a.px + sx;
 #pragma unroll
@@ -849,10 +871,9 @@ __global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel
       up[1] = ldg(a.u_in + V + q);
     }
   };
-  if (EARLY) load_rest();
+  if (EARLY && !ring_warp) load_rest();
   // 2. Halo ring.
-  constexpr int NRING = SW * SH - BX * BY;
-  for (int r = tid; r < NRING; r += NT) {
+  for (int r = tid; !RW && r < NRING; r += NT) {
     int lx, ly;
     ring_pos<R>(r, lx, ly);
     phi_global<P, NP, WALL>(a, wrap(x0 - R + lx, nx), wrap_y<WALL>(y0 - R + ly, ny),
@@ -863,7 +884,7 @@ __global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel
   // 3. Unequal densities: C_i on the tile and a ring of radius RC, then wall
   //    ghost rows of C repeat the adjacent fluid row.
   if constexpr (NU) {
-    for (int r = tid; r < CW * CH; r += NT) {
+    for (int r = tid; r < CW * CH; r += NT + 32 * RW) {
       const int cy = r / CW, cxl = r % CW;
       T ph[NP], lp[NP], cc[NP + 1], rho, hf[NP];
 #pragma unroll
@@ -882,7 +903,7 @@ __global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel
     }
     __syncthreads();
     if constexpr (WALL) {
-      for (int r = tid; r < CW * CH; r += NT) {
+      for (int r = tid; r < CW * CH; r += NT + 32 * RW) {
         const int cy = r / CW, cxl = r % CW;
         const int yg = y0 - RC + cy;
         if (yg < 0 || yg >= ny) {
@@ -896,6 +917,7 @@ __global__ void __launch_bounds__(NT, TileMin<P, NP, NU, G40>::CTAS) tile_kernel
     }
   }
 
+  if (ring_warp) return;
   // 4. Own node: stencils, C_i, forces, u, p.
   if (!EARLY) load_rest();
   NodeMac<P, NP> m;
@@ -1699,7 +1721,7 @@ namespace lbm {
 // FP32 grids of up to four waves of tiles on 152 SMs take the generic kernel:
 // its CTAs start their loads at once and overlap on an SM, where the pipelined
 // kernel's single CTA fetches its tensor maps and fills its stages first. us
-// per step, pipelined / generic: N = 3, 64^2 4.04 / 3.35, 256^2 5.29 / 4.45,
+// per step, pipelined / generic: N = 3, 64^2 4.04 / 3.08, 256^2 5.29 / 4.15,
 // 384^2 (576 tiles) 7.88 / 7.65; N = 5, 256^2 8.40 / 6.23, 384^2 13.1 / 11.0,
 // 512^2 (1024 tiles) 20.8 / 23.2. Grids that are not whole tiles, beyond that
 // line: 1501 x 997 (rows padded to 1504) N = 4 85.6 / 101, N = 2 42.0 / 54.2;
@@ -1744,6 +1766,14 @@ cudaError_t launch_tile_t(const Consts &c, const Grid &g, int cur, int mode,
     }
   }
   dim3 grid(tiles_x(g.nx), tiles_y(g.ny)), block(BX, BY);
+  if constexpr (P == LBM_FP32) {
+    constexpr int RW = NU ? 6 : 3;  // ring of 84 (radius 1) or 176 (2) positions
+    if (mode == MODE_STEP && g.ring_warps && g.grad_scheme == 0 &&
+        (long long)tiles_x(g.nx) * tiles_y(g.ny) <= 152 * ring_ctas(NP, NU)) {
+      tile_kernel<P, NP, NU, WALL, false, RW><<<grid, dim3(BX, BY + RW), 0, s>>>(a);
+      return cudaGetLastError();
+    }
+  }
   if (g.grad_scheme == 1)
     tile_kernel<P, NP, NU, WALL, true><<<grid, block, 0, s>>>(a);
   else
