@@ -227,6 +227,35 @@ __device__ __forceinline__ typename Prec<P>::T load_gm(const KArgs<P> &a, int k,
   return to_T(ldg(a.gm_in + ((size_t)(k - 1)) * a.V + q));
 }
 
+// FP32 <-> FP64 on the integer units, the same bits as the hardware's
+// conversions, for the start kernels, which are bound by the FP64 units (two
+// per SM) that those run on: three to five for each stored population. Values
+// outside the normal FP32 range (zero aside) take the hardware's. Not for the
+// output fields: 2048^2, N = 5 325 us with, 315 without, bound by memory.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+  const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u || m == 0)
+    return __hiloint2double((int)((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)),
+                            (int)(b << 29));
+  return (double)v;
+}
+// To nearest, ties to even, or (ODD) to odd: truncated, then the last bit set
+// if anything was cut off.
+template <bool ODD> __device__ __forceinline__ float narrow(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned m = hi & 0x7fffffffu, cut = lo & 0x1fffffffu;
+  if (m - 0x38100000u < 0x0fe00000u) {  // 2^-126 <= |v| < 2^128
+    const unsigned f = __funnelshift_l(lo, m - 0x38000000u, 3);
+    const unsigned r = ODD ? f | (cut != 0) : f + ((cut + 0x0fffffffu + (f & 1u)) >> 29);
+    return __uint_as_float((hi & 0x80000000u) | r);
+  }
+  if ((m | lo) == 0) return __uint_as_float(hi);
+  if (!ODD) return __double2float_rn(v);
+  const float t = __double2float_rz(v);
+  return (double)t == v ? t : __uint_as_float(__float_as_uint(t) | 1u);
+}
+
 // 16-bit forms: every moving population is stored relative to part of its
 // equilibrium (Eqs. 25, N25) evaluated at the node it was streamed from:
 // slot k of node y holds
@@ -1558,6 +1587,22 @@ __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
   }
 }
 
+// Store an FP64 value in a storage type with one rounding (to nearest, ties
+// to even). The 16-bit types go through FP32 rounded to odd (truncate, then
+// set the last bit if anything was cut off), which keeps the second rounding
+// exact: Boldo and Melquiond, "Emulation of FMA and correctly rounded sums:
+// proved algorithms using rounding to odd" (IEEE Trans. Computers, 2008),
+// for a target of at most 22 significant bits.
+template <typename S> __device__ __forceinline__ S store_once(double v);
+template <> __device__ __forceinline__ double store_once(double v) { return v; }
+template <> __device__ __forceinline__ float store_once(double v) { return narrow<false>(v); }
+template <> __device__ __forceinline__ __nv_bfloat16 store_once(double v) {
+  return to_S<__nv_bfloat16>(narrow<true>(v));
+}
+template <> __device__ __forceinline__ __half store_once(double v) {
+  return to_S<__half>(narrow<true>(v));
+}
+
 // ---------------------------------------------------------------------------
 // Initialisation: phi from c (inverse of Eqs. N2, N12), then h = h^eq and
 // g = g^eq at the stencil C_i.
@@ -1585,44 +1630,30 @@ __global__ void init_phi_kernel(const KArgs<P> a, const double *c,
     }
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      a.pp_out[(size_t)i * a.V + qp] = (T)ph[i];
+      a.pp_out[(size_t)i * a.V + qp] = store_once<T>(ph[i]);
       phid[(size_t)i * Vd + q] = ph[i];
     }
-    a.u_out[qp] = u ? (T)u[q] : T(0);
-    a.u_out[a.V + qp] = u ? (T)u[Vd + q] : T(0);
+    a.u_out[qp] = u ? store_once<T>(u[q]) : T(0);
+    a.u_out[a.V + qp] = u ? store_once<T>(u[Vd + q]) : T(0);
   }
 }
 
-// Store an FP64 value in a storage type with one rounding (to nearest, ties
-// to even). The 16-bit types go through FP32 rounded to odd (truncate, then
-// set the last bit if anything was cut off), which keeps the second rounding
-// exact: Boldo and Melquiond, "Emulation of FMA and correctly rounded sums:
-// proved algorithms using rounding to odd" (IEEE Trans. Computers, 2008),
-// for a target of at most 22 significant bits.
-template <typename S> __device__ __forceinline__ S store_once(double v);
-template <> __device__ __forceinline__ double store_once(double v) { return v; }
-template <> __device__ __forceinline__ float store_once(double v) {
-  return __double2float_rn(v);
-}
-__device__ __forceinline__ float float_round_odd(double v) {
-  const float t = __double2float_rz(v);
-  return (double)t == v ? t : __uint_as_float(__float_as_uint(t) | 1u);
-}
-template <> __device__ __forceinline__ __nv_bfloat16 store_once(double v) {
-  return to_S<__nv_bfloat16>(float_round_odd(v));
-}
-template <> __device__ __forceinline__ __half store_once(double v) {
-  return to_S<__half>(float_round_odd(v));
-}
+// Stored units of a moving population over its weight, s / w_k, for the faces
+// ([0]) and corners ([1]) of the velocity set.
+struct InitScale { double h[2], g[2]; };
 
 // Equilibrium start in FP64 for every storage form: phi (FP64, from
 // init_phi_kernel) and its Laplacian, C_i (Eqs. N17, N18), h^eq (Eq. N25) and g^eq
 // (Eq. 25) are computed in double with the constants `d`, and each stored
 // value is rounded once into its form. The 16-bit references (and the FP32
-// phi(t-1), u(t-1) they use) are those the step kernel decodes with.
+// phi(t-1), u(t-1) they use) are those the step kernel decodes with. Bound by
+// the FP64 units: conversions on the integer units, the scales divided once on
+// the host, a source's index and c_k.u formed once for g and all h^i. us, both
+// start kernels, before / after: 2048^2, N = 5, FP16 5580 / 4300, FP32 3770 /
+// 3640; 1024^2, N = 3, unequal, BF16 778 / 570.
 template <int P, int NP, bool WALL>
 __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
-                                const double *__restrict__ phid,
+                                const InitScale sc, const double *__restrict__ phid,
                                 const double *__restrict__ uin, double p0) {
   typedef typename Prec<P>::T T;
   typedef typename Prec<P>::Sm Sm;
@@ -1654,57 +1685,61 @@ __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
     const double ux = uin ? uin[qd] : 0.0, uy = uin ? uin[Vd + qd] : 0.0;
     const double uu = ux * ux + uy * uy;
     if constexpr (Prec<P>::REF) a.u_out[2 * V + q] = (T)p0;
-#pragma unroll
-    for (int k = 1; k < 9; ++k) {
-      const double cu = cx_of(k) * ux + cy_of(k) * uy;
-      const double geq =
-          w_of<double>(k) * (3.0 * p0 + rho * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu));
-      if constexpr (Prec<P>::MIX) {
-        const size_t qs = source_node<WALL>(x, y, k, nx, ny, a.px);
-        const T sux = a.u_out[qs], suy = a.u_out[V + qs];
-        // every source starts at p0 (stored as its p(t-1) above)
-        const T ref = Prec<P>::REF ? g_refp(cdotu(k, sux, suy), sux, suy, (T)p0,
-                                            a.rho_base * a.sg_st, T(3) * a.sg_st)
-                                   : T(0);
-        gm[(size_t)(k - 1) * V + q] =
-            store_once<Sm>(geq * (d.sg_st / w_of<double>(k)) - (double)ref);
-      } else
-        gm[(size_t)(k - 1) * V + q] = store_once<Sm>(geq);
-    }
+    double aC[NP], moving[NP];  // sum of the moving populations as stored
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
       double Ci = d.bulk * hf[i];
 #pragma unroll
       for (int j = 0; j < NP; ++j) Ci -= d.lam[i][j] * lp[j];
-      const double aC = d.a[i] * Ci;
-      double moving = 0.0;  // sum of the moving populations as stored
+      aC[i] = d.a[i] * Ci;
+      moving[i] = 0.0;
+    }
 #pragma unroll
-      for (int k = 1; k < 9; ++k) {
-        const double heq =
-            w_of<double>(k) * (aC + 3.0 * ph[i] * (cx_of(k) * ux + cy_of(k) * uy));
+    for (int k = 1; k < 9; ++k) {
+      const double cu = cx_of(k) * ux + cy_of(k) * uy;
+      const double geq =
+          w_of<double>(k) * (3.0 * p0 + rho * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu));
+      T scu = T(0);  // c_k.u(t-1) of slot k's source
+      size_t qs = 0;
+      if constexpr (Prec<P>::MIX) {
+        T ref = T(0);
+        if constexpr (Prec<P>::REF) {
+          qs = source_node<WALL>(x, y, k, nx, ny, a.px);
+          const T sux = a.u_out[qs], suy = a.u_out[V + qs];
+          scu = cdotu(k, sux, suy);
+          // every source starts at p0 (stored as its p(t-1) above)
+          ref = g_refp(scu, sux, suy, (T)p0, a.rho_base * a.sg_st, T(3) * a.sg_st);
+        }
+        gm[(size_t)(k - 1) * V + q] = store_once<Sm>(geq * sc.g[k > 4] - widen(ref));
+      } else
+        gm[(size_t)(k - 1) * V + q] = store_once<Sm>(geq);
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        const double heq = w_of<double>(k) * (aC[i] + 3.0 * ph[i] * cu);
         if constexpr (Prec<P>::MIX) {
-          const size_t qs = source_node<WALL>(x, y, k, nx, ny, a.px);
-          const T ref = Prec<P>::REF ? adv_units(cdotu(k, a.u_out[qs], a.u_out[V + qs]),
-                                                 a.pp_out[(size_t)i * V + qs], T(3) * a.sh_st)
+          const T ref = Prec<P>::REF ? adv_units(scu, a.pp_out[(size_t)i * V + qs], T(3) * a.sh_st)
                                      : T(0);
-          const Sm sv = store_once<Sm>(heq * (d.sh_st / w_of<double>(k)) - (double)ref);
+          const Sm sv = store_once<Sm>(heq * sc.h[k > 4] - widen(ref));
           hm[((size_t)(i * 8 + k - 1)) * V + q] = sv;
           const T dec = Prec<P>::REF ? __fadd_rn(to_T(sv), ref) : to_T(sv);
-          moving += (double)(w_of<T>(k) * a.sh_ld) * (double)dec;
+          moving[i] += widen(w_of<T>(k) * a.sh_ld) * widen(dec);
         } else {
           const Sm hv = store_once<Sm>(heq);
           hm[((size_t)(i * 8 + k - 1)) * V + q] = hv;
-          moving += (double)hv;
+          moving[i] += widen(hv);
         }
       }
-      // FP64: h_0 = h_0^eq. Other forms: d_0 = h_0 - phi(t-1) with phi(t-1)
-      // the stored (rounded) phi, so that phi(t-1) + d_0 + sum_{k>=1} h_k is
-      // phi up to the rounding of d_0.
+    }
+    // FP64: h_0 = h_0^eq. Other forms: d_0 = h_0 - phi(t-1) with phi(t-1)
+    // the stored (rounded) phi, so that phi(t-1) + d_0 + sum_{k>=1} h_k is
+    // phi up to the rounding of d_0.
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
       if constexpr (P == LBM_FP64)
-        h0[(size_t)i * V + q] = ph[i] + (w_of<double>(0) - 1.0) * aC;
+        h0[(size_t)i * V + q] = ph[i] + (w_of<double>(0) - 1.0) * aC[i];
       else
         h0[(size_t)i * V + q] =
-            store_once<T>((ph[i] - (double)a.pp_out[(size_t)i * V + q]) - moving);
+            store_once<T>((ph[i] - widen(a.pp_out[(size_t)i * V + q])) - moving[i]);
     }
   }
 }
@@ -1867,10 +1902,12 @@ cudaError_t launch_init_np(const Consts &c, const Grid &g, int cur,
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const KArgs<LBM_FP64> d = make_args<LBM_FP64>(c, g, cur ^ 1, MODE_STEP, Outputs{});
+  const InitScale sc = {{d.sh_st / w_of<double>(1), d.sh_st / w_of<double>(5)},
+                        {d.sg_st / w_of<double>(1), d.sg_st / w_of<double>(5)}};
   if (wall)
-    init_pop_kernel<P, NP, true><<<(unsigned)blocks, threads, 0, s>>>(a, d, g.scratch, uin, p0);
+    init_pop_kernel<P, NP, true><<<(unsigned)blocks, threads, 0, s>>>(a, d, sc, g.scratch, uin, p0);
   else
-    init_pop_kernel<P, NP, false><<<(unsigned)blocks, threads, 0, s>>>(a, d, g.scratch, uin, p0);
+    init_pop_kernel<P, NP, false><<<(unsigned)blocks, threads, 0, s>>>(a, d, sc, g.scratch, uin, p0);
   return cudaGetLastError();
 }
 
