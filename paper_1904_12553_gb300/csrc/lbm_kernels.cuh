@@ -835,13 +835,20 @@ template <int P, int NP, bool NU, bool G40> struct TileMin {
 // the ring's is then off the chain, for ring_ctas CTAs per SM at the registers
 // that this takes. us per step, with / without: N = 3, 64^2 3.08 / 3.29, 256^2
 // 4.15 / 4.50; N = 5, 128^2 3.97 / 4.51; unequal densities: N = 3 with walls,
-// 150^2 3.79 / 4.45, 256^2 5.07 / 5.73; N = 5 with walls, 150^2 5.23 / 5.71.
+// 150^2 3.79 / 4.45, 256^2 5.07 / 5.73; N = 5 with walls, 150^2 5.23 / 5.71;
+// Eq. N40: N = 2, 150^2 2.88 / 3.35, N = 3, 256^2 4.68 / 4.80, unequal, N = 3,
+// 150^2 4.13 / 4.99, N = 5, 200 x 150 5.71 / 6.55.
 // Beyond one wave the occupancy it gives up costs more: unequal N = 2, 400 x
 // 200 (325 tiles), 7.96 with 4 warps in 3 CTAs / 6.99.
-constexpr int ring_ctas(int NP, bool NU) { return NP <= (NU ? 2 : 3) ? 2 : 1; }
+constexpr int ring_ctas(int NP, bool NU, bool G40) {
+  return NP <= (NU && G40 ? 0 : NU || G40 ? 2 : 3) ? 2 : 1;
+}
+constexpr int ring_rw(bool NU, bool G40) {  // ring of radius 1, 2 or 3: 84, 176 or 276 positions
+  return NU && G40 ? 9 : NU || G40 ? 6 : 3;
+}
 template <int P, int NP, bool NU, bool WALL, bool G40, int RW = 0>
 __global__ void __launch_bounds__(NT + 32 * RW,
-                                  RW ? ring_ctas(NP, NU) : TileMin<P, NP, NU, G40>::CTAS)
+                                  RW ? ring_ctas(NP, NU, G40) : TileMin<P, NP, NU, G40>::CTAS)
     tile_kernel(const KArgs<P> a) {
   constexpr bool EARLY = TileMin<P, NP, NU, G40>::EARLY || RW;
   typedef typename Prec<P>::T T;
@@ -1802,10 +1809,14 @@ cudaError_t launch_tile_t(const Consts &c, const Grid &g, int cur, int mode,
   }
   dim3 grid(tiles_x(g.nx), tiles_y(g.ny)), block(BX, BY);
   if constexpr (P == LBM_FP32) {
-    constexpr int RW = NU ? 6 : 3;  // ring of 84 (radius 1) or 176 (2) positions
-    if (mode == MODE_STEP && g.ring_warps && g.grad_scheme == 0 &&
-        (long long)tiles_x(g.nx) * tiles_y(g.ny) <= 152 * ring_ctas(NP, NU)) {
-      tile_kernel<P, NP, NU, WALL, false, RW><<<grid, dim3(BX, BY + RW), 0, s>>>(a);
+    const bool g40 = g.grad_scheme == 1;
+    if (mode == MODE_STEP && g.ring_warps &&
+        (long long)tiles_x(g.nx) * tiles_y(g.ny) <= 152 * ring_ctas(NP, NU, g40)) {
+      constexpr int RW = ring_rw(NU, false), RW40 = ring_rw(NU, true);
+      if (g40)
+        tile_kernel<P, NP, NU, WALL, true, RW40><<<grid, dim3(BX, BY + RW40), 0, s>>>(a);
+      else
+        tile_kernel<P, NP, NU, WALL, false, RW><<<grid, dim3(BX, BY + RW), 0, s>>>(a);
       return cudaGetLastError();
     }
   }

@@ -47,3 +47,27 @@ def test_ring_warps_match_generic(N, nx, ny, wall, unequal):
             continue
         bound = max(1e-6 * np.abs(y).max(), 2 * np.abs(y - z).max())
         assert np.abs(x - y).max() <= bound, k
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 1), (33, 9), (150, 37), (256, 152), (257, 152), (608, 128)])
+@pytest.mark.parametrize("N", [2, 3, 4, 5])
+@pytest.mark.parametrize("wall", [0, 1])
+@pytest.mark.parametrize("unequal", [0, 1])
+def test_ring_warps_mixed_gradients(N, nx, ny, wall, unequal):
+    """Eq. N40: rings of radius 2 and 3, by the same comparison."""
+    seed = 17 * N + nx + 3 * ny + wall
+    rho = [1.0 + 0.5 * k for k in range(N)] if unequal else None
+
+    def case(precision):
+        return W.random_smooth(seed, N, nx, ny, rho=rho, wall_y=wall, amp_u=0.01, sigma=1e-3,
+                               grad_scheme=1, precision=precision)
+
+    a = gpu_run(case("fp32"), 8)
+    b = gpu_run(case("fp32"), 8, kernel="generic")
+    e = gpu_run(case("fp64"), 8, kernel="generic")
+    for k in ("phi", "u", "p"):
+        x, y, z = (np.asarray(m[k]) for m in (a, b, e))
+        if np.array_equal(x, y, equal_nan=True):
+            continue
+        bound = max(1e-6 * np.abs(y).max(), 2 * np.abs(y - z).max())
+        assert np.abs(x - y).max() <= bound, k
