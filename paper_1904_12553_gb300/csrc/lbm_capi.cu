@@ -168,6 +168,14 @@ lbm_status validate(const lbm_nphase_params *p) {
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
+// LBM_NPHASE_KERNEL: "generic" selects the generic tile kernels everywhere,
+// "pipelined" the TMA kernels at every size; else the rules below.
+bool kernel_env(const char *name) {
+  const char *v = getenv("LBM_NPHASE_KERNEL");
+  return v && strcmp(v, name) == 0;
+}
+bool tma_allowed() { return !kernel_env("generic"); }
+
 struct Layout {
   size_t h0, hm, gm, phi_prev, u_prev, stage, red, red_out, err, total;
 };
@@ -182,21 +190,21 @@ int uplanes(const lbm_nphase_params *p) {
   return dims(p) + (p->precision == LBM_MIX_BF16 || p->precision == LBM_MIX_FP16 ? 1 : 0);
 }
 
-// Row pitch of the state's planes. The pipelined D2Q9 kernels need rows of
-// whole 16 bytes: grids they can serve (FP32 and 16-bit forms, equal
-// densities, central scheme) are padded to a multiple of 8 nodes, at most 7
-// nodes per row. FP32, us per step on the generic kernel, dense -> padded:
-// see pipelined_pays.
+// Row pitch of the state's planes: FP32 D2Q9 grids that the pipelined kernel
+// serves have their rows padded to a multiple of 8 nodes for its TMA loads.
+// The others stay dense: a padded row costs the generic kernel up to a quarter
+// (33 x 40000, N = 5 172 -> 216 us per step) and a narrow grid its memory.
 int pitch(const lbm_nphase_params *p, bool pad) {
-  if (!pad || p->lattice != 0 || p->precision != LBM_FP32 || p->grad_scheme != 0) return p->nx;
+  if (!pad || !tma_allowed() || p->lattice != 0 || p->precision != LBM_FP32 || p->grad_scheme != 0) return p->nx;
   for (int k = 1; k < p->N; ++k)
     if (p->rho[k] != p->rho[0]) return p->nx;
+  if (!lbm::tma_pays(p->N, p->nx, p->ny) && !kernel_env("pipelined")) return p->nx;
   return (p->nx + 7) / 8 * 8;
 }
 
-Layout layout(const lbm_nphase_params *p, bool pad) {
+Layout layout(const lbm_nphase_params *p, int px) {
   const size_t Vd = (size_t)p->nx * p->ny * depth(p);
-  const size_t V = (size_t)pitch(p, pad) * p->ny * depth(p);
+  const size_t V = (size_t)px * p->ny * depth(p);
   const int NP = p->N - 1, QM = moving_dirs(p), D = dims(p), UP = uplanes(p);
   const size_t sT = p->precision == LBM_FP64 ? 8 : 4;
   const size_t sS = p->precision == LBM_FP64 ? 8 : (p->precision == LBM_FP32 ? 4 : 2);
@@ -246,14 +254,6 @@ lbm::EncodeTiledFn tensor_map_encoder() {
       cudaGetLastError();
   }
   return fn;
-}
-
-// Which step kernel to use: the pipelined TMA kernel where it applies
-// (default), or the generic tile kernel everywhere when the environment
-// variable LBM_NPHASE_KERNEL is "generic".
-bool tma_allowed() {
-  const char *v = getenv("LBM_NPHASE_KERNEL");
-  return !(v && strcmp(v, "generic") == 0);
 }
 
 // Device error word: read and clear. Returns LBM_ETIMEOUT if a kernel's
@@ -432,7 +432,7 @@ lbm_status lbm_nphase_create(const lbm_nphase_params *p, void *ws,
 }  // extern "C"
 
 size_t lbm::workspace_bytes(const lbm_nphase_params *p, bool pad) {
-  return validate(p) == LBM_OK ? layout(p, pad).total : 0;
+  return validate(p) == LBM_OK ? layout(p, pitch(p, pad)).total : 0;
 }
 
 lbm_status lbm::create(const lbm_nphase_params *p, void *ws, size_t bytes, void *stream, bool pad,
@@ -443,7 +443,10 @@ lbm_status lbm::create(const lbm_nphase_params *p, void *ws, size_t bytes, void 
   lbm_status st = lbm_nphase_derive(p, &m);
   if (st != LBM_OK) return st;
   if (!ws || ((uintptr_t)ws & 255u)) return LBM_EINVAL;
-  const Layout L = layout(p, pad);
+  // a workspace that holds the dense state only is served too (generic kernel)
+  int px = pitch(p, pad);
+  if (bytes < layout(p, px).total) px = p->nx;
+  const Layout L = layout(p, px);
   if (bytes < L.total) return LBM_ENOMEM;
   lbm_nphase_t *h = new (std::nothrow) lbm_nphase_t;
   if (!h) return LBM_ENOMEM;
@@ -500,7 +503,7 @@ lbm_status lbm::create(const lbm_nphase_params *p, void *ws, size_t bytes, void 
   g.ny = p->ny;
   g.nz = depth(p);
   g.lattice = p->lattice;
-  g.px = pitch(p, pad);
+  g.px = px;
   g.V = (size_t)g.px * p->ny * g.nz;
   char *base = (char *)ws;
   const size_t sT = h->prec == LBM_FP64 ? 8 : 4;
@@ -532,8 +535,7 @@ lbm_status lbm::create(const lbm_nphase_params *p, void *ws, size_t bytes, void 
              (size_t)p->nx * p->ny * sT < ((size_t)1 << 32);
   g.march3 = g.split3 && !h->nonunif;
   g.ring_warps = tma_allowed();
-  const char *kv = getenv("LBM_NPHASE_KERNEL");
-  g.tma_all = kv && strcmp(kv, "pipelined") == 0;
+  g.tma_all = kernel_env("pipelined");
   g.tma3 = g.march3 && h->prec == LBM_FP32 &&
            lbm::encode_tma3_f32(k, g, tensor_map_encoder());
   if (tma_allowed() && !h->nonunif && p->grad_scheme == 0 && p->lattice == 0) {

@@ -60,7 +60,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType,
 struct Grid {
   int nx, ny, nz;   // nz = 1 for D2Q9
   int lattice;      // 0 D2Q9, 1 D3Q15
-  int px;           // row pitch in nodes (nx, or nx rounded up to 8)
+  int px;           // row pitch in nodes (nx, or rounded up to 8: see pitch())
   size_t V;         // plane stride px * ny * nz
   void *h0[2];      // rest slots: h^i_0 (FP64) or h^i_0 - phi_i(t-1): [N-1][V]
   void *hm[2];      // moving populations h^i_k, k = 1..8: [N-1][8][V]
@@ -123,6 +123,30 @@ inline int tiles_y(int ny) { return (ny + BY - 1) / BY; }
 inline int tiles3_x(int nx) { return (nx + 31) / 32; }
 inline int tiles3_y(int ny) { return (ny + 3) / 4; }
 inline int tiles3_z(int nz) { return (nz + 1) / 2; }
+inline long long tiles_of(int nx, int ny) { return (long long)tiles_x(nx) * tiles_y(ny); }
+// FP32 D2Q9 grids (equal densities, central scheme): the pipelined kernel, or
+// the generic one, whose CTAs start their loads at once and overlap on an SM
+// where the pipelined kernel's single CTA fetches its tensor maps and fills its
+// stages first. The line lies at six to eight waves of tiles on 152 SMs, by
+// phases (pipelined / generic, us per step, chains of steps):
+//   N = 2: 513^2 (1105 tiles) 9.6 / 9.0, 640 x 512 (1280) 10.0 / 10.8
+//   N = 3: 512 x 400 (800) 10.4 / 9.6, 512^2 (1024) 11.6 / 11.8
+//   N = 4: 512^2 16.7 / 15.6, 640 x 480 (1200) 17.8 / 18.8
+//   N = 5: 512 x 400 17.4 / 16.3, 512^2 20.0 / 21.6
+// and 2048^2 109 / 135, 161 / 211, 221 / 260, 265 / 360 at N = 2..5. Tiles
+// with idle lanes fill a whole stage all the same: grids up to 63 wide (57 x
+// 40000, N = 5 267 / 244; 8 x 40000, N = 3 78 / 37) or with fewer than 60% of
+// the lanes in use (20001 x 9, N = 4 18.0 / 14.4; N = 4 also 65 x 5000, 68%,
+// 29.7 / 26.5) stay on the generic kernel.
+inline bool tma_pays(int N, int nx, int ny) {
+  const long long t = tiles_of(nx, ny), line = N == 2 ? 1216 : N == 4 ? 1140 : 912;
+  return nx >= 64 && t > line && (long long)nx * ny * 100 >= t * 256 * (N == 4 ? 70 : 60);
+}
+// N = 3: three stages of 49 KB and one CTA per SM; two and two CTAs hold 216 KB,
+// which leaves L1 too little for the stores. us per step, 2 stages x 2 CTAs / 2 x
+// 1 / 3 x 1 / 4 x 1: 2048^2 213 / 184 / 165 / 215, 1504 x 1000 69.1 / 68.2 / 60.3 /
+// 67.1, 1024^2 48.8 / 49.0 / 45.3 / 46.2.
+inline bool tma_three_stages(int, int) { return true; }
 // CTAs of the generic step / moments / diagnostics kernel of a grid
 inline size_t tiles_total(int lattice, int nx, int ny, int nz) {
   return lattice == 1 ? (size_t)tiles3_x(nx) * tiles3_y(ny) * tiles3_z(nz)

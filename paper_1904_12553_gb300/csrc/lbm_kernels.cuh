@@ -1127,7 +1127,8 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map,
       : "memory");
 }
 
-template <int P, int NP> struct TmaStage {
+// ST: stages of one CTA (tma_three_stages)
+template <int P, int NP, int ST = TmaGeom<P>::S> struct TmaStage {
   typedef typename Prec<P>::T T;
   typedef typename Prec<P>::Sm Sm;
   typedef TmaGeom<P> G;
@@ -1160,12 +1161,8 @@ template <int P, int NP> struct TmaStage {
   static constexpr uint32_t YTX =
       (uint32_t)((size_t)8 * NP * G::WM * sizeof(Sm) + (size_t)2 * NP * G::WR * sizeof(T));
   static constexpr size_t SPHI = al((size_t)NP * (G::TBY + 2) * (BX + 2) * sizeof(T));
-  // Stages. FP32, N = 3: three of 49 KB and one CTA per SM; two and two CTAs
-  // hold 216 KB, which leaves L1 too little for the stores. us per step, 2
-  // stages x 2 CTAs / 2 x 1 / 3 x 1 / 4 x 1: 2048^2 213 / 184 / 165 / 215,
-  // 1504 x 1000 69.1 / 68.2 / 60.3 / 67.1, 1024^2 48.8 / 49.0 / 45.3 / 46.2.
-  static constexpr int S = G::WIDE && NP == 2 ? 3 : G::S;
-  static constexpr int CTAS = G::WIDE && NP == 2 ? 1 : 8;  // most per SM
+  static constexpr int S = ST;
+  static constexpr int CTAS = ST > G::S ? 1 : 8;  // most per SM
   // FP32: two phi tiles (one barrier per tile, below); 16-bit forms: one
   static constexpr int NPHI = G::WIDE ? 2 : 1;
   static constexpr size_t SMEM = S * BYTES + NPHI * SPHI + 64;
@@ -1197,14 +1194,14 @@ __device__ __forceinline__ void ring_pos_1(int r, int &lx, int &ly) {
 // ghost row is the adjacent row; a source behind a wall is the node
 // itself): one branch-free path for all tiles. Other grids take a general
 // path that reads wrapped positions from global memory.
-template <int P, int NP, bool WALL, bool WHOLE>
+template <int P, int NP, bool WALL, bool WHOLE, int ST>
 __global__ void __launch_bounds__(TmaGeom<P>::NTH, TmaGeom<P>::WIDE ? 1 : 2)
     tile_kernel_tma(const KArgs<P> a, const __grid_constant__ TmaMaps maps,
                     int ntx, int ntiles) {
   typedef typename Prec<P>::T T;
   typedef typename Prec<P>::Sm Sm;
   typedef TmaGeom<P> G;
-  typedef TmaStage<P, NP> St;
+  typedef TmaStage<P, NP, ST> St;
   constexpr int S = St::S;
   constexpr int TBY = G::TBY;
   constexpr int SW = BX + 2, SH = TBY + 2, PL = SW * SH;
@@ -1760,18 +1757,34 @@ namespace lbm {
 // ---------------------------------------------------------------------------
 // Host-side launchers for one precision.
 // ---------------------------------------------------------------------------
-// FP32 grids of up to four waves of tiles on 152 SMs take the generic kernel:
-// its CTAs start their loads at once and overlap on an SM, where the pipelined
-// kernel's single CTA fetches its tensor maps and fills its stages first. us
-// per step, pipelined / generic: N = 3, 64^2 4.04 / 3.08, 256^2 5.29 / 4.15,
-// 384^2 (576 tiles) 7.88 / 7.65; N = 5, 256^2 8.40 / 6.23, 384^2 13.1 / 11.0,
-// 512^2 (1024 tiles) 20.8 / 23.2. Grids that are not whole tiles, beyond that
-// line: 1501 x 997 (rows padded to 1504) N = 4 85.6 / 101, N = 2 42.0 / 54.2;
-// 1200 x 900 N = 5 141 -> 81.6 with the wrapped column and row of overhanging
-// tiles staged. The 16-bit forms' decode makes the generic
-// kernel slower at every size (BF16 N = 3, 128^2 4.9 / 6.6).
-template <int P> inline bool pipelined_pays(const Grid &g) {
-  return P != LBM_FP32 || g.tma_all || (long long)tiles_x(g.nx) * tiles_y(g.ny) > 4 * 152;
+// The pipelined kernel's persistent CTAs. FP32 grids take it where tma_pays
+// says so; the 16-bit forms' decode makes the generic kernel slower at every
+// size (BF16 N = 3, 128^2 4.9 / 6.6 us per step).
+template <int P, int NP, bool WALL, int ST>
+cudaError_t launch_tma_t(const KArgs<P> &a, const Grid &g, int cur, cudaStream_t s) {
+  typedef TmaStage<P, NP, ST> St;
+  constexpr int TBY = TmaGeom<P>::TBY;
+  const bool whole = g.nx % BX == 0 && g.ny % TBY == 0 && g.nx > BX && g.ny > TBY;
+  auto kern =
+      whole ? tile_kernel_tma<P, NP, WALL, true, ST> : tile_kernel_tma<P, NP, WALL, false, ST>;
+  static int max_ctas[2] = {0, 0};  // per instantiation: resident CTAs on the GPU
+  int &mc = max_ctas[whole ? 1 : 0];
+  if (mc == 0) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)St::SMEM);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0, dev = 0, sms = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TmaGeom<P>::NTH, St::SMEM);
+    if (e != cudaSuccess) return e;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    per_sm = per_sm > St::CTAS ? St::CTAS : per_sm;
+    mc = (per_sm > 0 ? per_sm : 1) * sms;
+  }
+  const int ntx = tiles_x(g.nx), ntiles = ntx * ((g.ny + TBY - 1) / TBY);
+  const int grid = ntiles < mc ? ntiles : mc;
+  kern<<<grid, dim3(BX, TBY), St::SMEM, s>>>(a, *(const TmaMaps *)&g.tma[cur], ntx, ntiles);
+  return cudaGetLastError();
 }
 
 template <int P, int NP, bool NU, bool WALL>
@@ -1781,30 +1794,11 @@ cudaError_t launch_tile_t(const Consts &c, const Grid &g, int cur, int mode,
     if (mode == MODE_STEP && g.step64) return launch_step64<NP, NU, WALL>(c, g, cur, s);
   const KArgs<P> a = make_args<P>(c, g, cur, mode, o);
   if constexpr (P != LBM_FP64 && !NU) {
-    if (mode == MODE_STEP && g.use_tma && g.grad_scheme == 0 && pipelined_pays<P>(g)) {
-      typedef TmaStage<P, NP> St;
-      constexpr int TBY = TmaGeom<P>::TBY;
-      const bool whole = g.nx % BX == 0 && g.ny % TBY == 0 && g.nx > BX && g.ny > TBY;
-      auto kern = whole ? tile_kernel_tma<P, NP, WALL, true> : tile_kernel_tma<P, NP, WALL, false>;
-      static int max_ctas[2] = {0, 0};  // per instantiation: resident CTAs on the GPU
-      int &mc = max_ctas[whole ? 1 : 0];
-      if (mc == 0) {
-        cudaError_t e = cudaFuncSetAttribute(
-            kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)St::SMEM);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, dev = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TmaGeom<P>::NTH,
-                                                          St::SMEM);
-        if (e != cudaSuccess) return e;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        per_sm = per_sm > St::CTAS ? St::CTAS : per_sm;
-        mc = (per_sm > 0 ? per_sm : 1) * sms;
-      }
-      const int ntx = tiles_x(g.nx), ntiles = ntx * ((g.ny + TBY - 1) / TBY);
-      const int grid = ntiles < mc ? ntiles : mc;
-      kern<<<grid, dim3(BX, TBY), St::SMEM, s>>>(a, *(const TmaMaps *)&g.tma[cur], ntx, ntiles);
-      return cudaGetLastError();
+    if (mode == MODE_STEP && g.use_tma &&
+        (P != LBM_FP32 || g.tma_all || tma_pays(c.N, g.nx, g.ny))) {
+      if constexpr (P == LBM_FP32 && NP == 2)
+        if (tma_three_stages(g.nx, g.ny)) return launch_tma_t<P, NP, WALL, 3>(a, g, cur, s);
+      return launch_tma_t<P, NP, WALL, TmaGeom<P>::S>(a, g, cur, s);
     }
   }
   dim3 grid(tiles_x(g.nx), tiles_y(g.ny)), block(BX, BY);
