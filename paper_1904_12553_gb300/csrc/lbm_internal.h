@@ -142,11 +142,16 @@ inline bool tma_pays(int N, int nx, int ny) {
   const long long t = tiles_of(nx, ny), line = N == 2 ? 1216 : N == 4 ? 1140 : 912;
   return nx >= 64 && t > line && (long long)nx * ny * 100 >= t * 256 * (N == 4 ? 70 : 60);
 }
-// N = 3: three stages of 49 KB and one CTA per SM; two and two CTAs hold 216 KB,
-// which leaves L1 too little for the stores. us per step, 2 stages x 2 CTAs / 2 x
-// 1 / 3 x 1 / 4 x 1: 2048^2 213 / 184 / 165 / 215, 1504 x 1000 69.1 / 68.2 / 60.3 /
-// 67.1, 1024^2 48.8 / 49.0 / 45.3 / 46.2.
-inline bool tma_three_stages(int, int) { return true; }
+// N = 3: three stages of 49 KB and one CTA per SM where the state is far beyond
+// L2, else two and two CTAs (216 KB, which leave L1 little for the stores, but
+// twice the warps). us per step, 3 x 1 / 2 x 2: 256 x 1600 (1600 tiles) 21.1 /
+// 16.5, 768^2 (2304) 28.0 / 24.0, 1200 x 900 (4294) 55.1 / 48.4, 1501 x 997
+// (5875) 61.8 / 65.0, 96 x 40000 163 / 190, 2048^2 161 / 206; narrow rows of
+// whole 32 bytes keep two longer: 64 x 40000 115 / 107, 72 x 40000 168 / 147
+// (73 x 40000 173 / 203). 2 x 1 and 4 x 1 are slower than both at 2048^2.
+inline bool tma_three_stages(int nx, int ny) {
+  return tiles_of(nx, ny) > 33 * 152 && (nx >= 96 || nx % 8 != 0);
+}
 // CTAs of the generic step / moments / diagnostics kernel of a grid
 inline size_t tiles_total(int lattice, int nx, int ny, int nz) {
   return lattice == 1 ? (size_t)tiles3_x(nx) * tiles3_y(ny) * tiles3_z(nz)

@@ -1,5 +1,5 @@
-"""FP32 grids on either side of the rule that chooses the pipelined kernel,
-against the generic kernel: the same step and arithmetic, within
+"""FP32 grids on either side of the rules that choose the pipelined kernel and
+its stages, against the generic kernel: the same step and arithmetic, within
 1e-6 of the largest value (the bound of the pipelined kernel's other
 comparisons)."""
 import pytest
@@ -19,6 +19,15 @@ torch = pytest.importorskip("torch")
 def test_either_side_of_the_line(N, nx, ny, wall):
     w = case(N, nx, ny, wall)
     check(gpu_run(w, 12), gpu_run(w, 12, kernel="generic"))
+
+
+# N = 3: two stages and two CTAs per SM, and from 5017 tiles three and one
+@pytest.mark.parametrize("nx,ny", [(1216, 1056), (1248, 1040), (1504, 1000), (1501, 1003),
+                                   (97, 10037)])
+@pytest.mark.parametrize("wall", [0, 1])
+def test_stages_of_three_phases(nx, ny, wall):
+    w = case(3, nx, ny, wall)
+    check(gpu_run(w, 6), gpu_run(w, 6, kernel="generic"))
 
 
 # narrow grids, and grids with few lanes in use: the generic kernel on dense rows
