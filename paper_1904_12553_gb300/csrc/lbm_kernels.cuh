@@ -825,7 +825,10 @@ __device__ __forceinline__ void phi_global(const KArgs<P> &a, int sx, int sy,
 template <int P, int NP, bool NU, bool G40> struct TileMin {
   static constexpr bool F32 = P == LBM_FP32;
   static constexpr bool EARLY = F32 && !NU && NP != 1;
-  static constexpr int CTAS = !F32 ? 0 : (NP == 4 ? 2 : (NP == 1 || (NU && !G40 && NP == 2) ? 4 : 3));
+  static constexpr int CTAS =
+      P == LBM_FP64 ? 0
+      : F32         ? (NP == 4 ? 2 : (NP == 1 || (NU && !G40 && NP == 2) ? 4 : 3))
+                    : (NP == 1 ? 4 : NP == 2 ? 3 : NP == 4 ? 2 : 0);
 };
 
 // RW > 0 (FP32 step): that many more warps sum phi on the halo ring, one
@@ -893,9 +896,9 @@ __global__ void __launch_bounds__(NT + 32 * RW,
           node_phi<P>(hreg[i][0], &hreg[i][1], pp, perr[i], a.sh_ld);
     }
   }
-  const size_t q = (size_t)(active ? gy : 0) * a.px + (active ? gx : 0);
   T g[9], up[2];
   auto load_rest = [&] {  // the node's NS populations and u(t-1)
+    const size_t q = (size_t)(active ? gy : 0) * a.px + (active ? gx : 0);
     if (active) {
       load_g_node<P, WALL>(a, gx, gy, q, g);
     } else {
@@ -955,6 +958,7 @@ __global__ void __launch_bounds__(NT + 32 * RW,
 
   if (ring_warp) return;
   // 4. Own node: stencils, C_i, forces, u, p.
+  const size_t q = (size_t)(active ? gy : 0) * a.px + (active ? gx : 0);
   if (!EARLY) load_rest();
   NodeMac<P, NP> m;
   node_macros<P, NP, NU, SW, CW, G40>(a, &sphi[0][0], SH * SW, &sC[0][0],
