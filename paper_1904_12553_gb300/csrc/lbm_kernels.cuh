@@ -1628,7 +1628,7 @@ __global__ void init_phi_kernel(const KArgs<P> a, const double *c,
   const size_t Vd = (size_t)a.nx * a.ny;  // dense inputs and phid, pitched state
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < Vd;
        q += (size_t)gridDim.x * blockDim.x) {
-    const size_t qp = q / a.nx * a.px + q % a.nx;
+    const size_t qp = a.px == a.nx ? q : q / a.nx * a.px + q % a.nx;
     const double cN = c[(size_t)NP * Vd + q];
     double ph[NP];
 #pragma unroll
@@ -1658,8 +1658,11 @@ struct InitScale { double h[2], g[2]; };
 // the FP64 units: conversions on the integer units, the scales divided once on
 // the host, a source's index and c_k.u formed once for g and all h^i. us, both
 // start kernels, before / after: 2048^2, N = 5, FP16 5580 / 4300, FP32 3770 /
-// 3640; 1024^2, N = 3, unequal, BF16 778 / 570.
-template <int P, int NP, bool WALL>
+// 3640; 1024^2, N = 3, unequal, BF16 778 / 570. REST: without a velocity (uin is
+// null), compiled apart for two phases in FP32, where it leaves little FP64 work
+// (us, 1280 x 1024: 395 in one kernel with the moving start, 215 apart, with the
+// hardware's conversions, which are the fewer instructions there).
+template <int P, int NP, bool WALL, bool REST>
 __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
                                 const InitScale sc, const double *__restrict__ phid,
                                 const double *__restrict__ uin, double p0) {
@@ -1690,7 +1693,7 @@ __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
     }
     double cc[NP + 1], rho, hf[NP];
     local_algebra<LBM_FP64, NP>(d, ph, cc, rho, hf);
-    const double ux = uin ? uin[qd] : 0.0, uy = uin ? uin[Vd + qd] : 0.0;
+    const double ux = !REST && uin ? uin[qd] : 0.0, uy = !REST && uin ? uin[Vd + qd] : 0.0;
     const double uu = ux * ux + uy * uy;
     if constexpr (Prec<P>::REF) a.u_out[2 * V + q] = (T)p0;
     double aC[NP], moving[NP];  // sum of the moving populations as stored
@@ -1720,7 +1723,7 @@ __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
         }
         gm[(size_t)(k - 1) * V + q] = store_once<Sm>(geq * sc.g[k > 4] - widen(ref));
       } else
-        gm[(size_t)(k - 1) * V + q] = store_once<Sm>(geq);
+        gm[(size_t)(k - 1) * V + q] = REST ? (Sm)geq : store_once<Sm>(geq);
 #pragma unroll
       for (int i = 0; i < NP; ++i) {
         const double heq = w_of<double>(k) * (aC[i] + 3.0 * ph[i] * cu);
@@ -1732,9 +1735,9 @@ __global__ void init_pop_kernel(const KArgs<P> a, const KArgs<LBM_FP64> d,
           const T dec = Prec<P>::REF ? __fadd_rn(to_T(sv), ref) : to_T(sv);
           moving[i] += widen(w_of<T>(k) * a.sh_ld) * widen(dec);
         } else {
-          const Sm hv = store_once<Sm>(heq);
+          const Sm hv = REST ? (Sm)heq : store_once<Sm>(heq);
           hm[((size_t)(i * 8 + k - 1)) * V + q] = hv;
-          moving[i] += widen(hv);
+          moving[i] += REST ? (double)hv : widen(hv);
         }
       }
     }
@@ -1913,10 +1916,11 @@ cudaError_t launch_init_np(const Consts &c, const Grid &g, int cur,
   const KArgs<LBM_FP64> d = make_args<LBM_FP64>(c, g, cur ^ 1, MODE_STEP, Outputs{});
   const InitScale sc = {{d.sh_st / w_of<double>(1), d.sh_st / w_of<double>(5)},
                         {d.sg_st / w_of<double>(1), d.sg_st / w_of<double>(5)}};
-  if (wall)
-    init_pop_kernel<P, NP, true><<<(unsigned)blocks, threads, 0, s>>>(a, d, sc, g.scratch, uin, p0);
-  else
-    init_pop_kernel<P, NP, false><<<(unsigned)blocks, threads, 0, s>>>(a, d, sc, g.scratch, uin, p0);
+  constexpr bool APART = P == LBM_FP32 && NP == 1;
+  auto kern = wall ? init_pop_kernel<P, NP, true, false> : init_pop_kernel<P, NP, false, false>;
+  if (APART && !uin)
+    kern = wall ? init_pop_kernel<P, NP, true, APART> : init_pop_kernel<P, NP, false, APART>;
+  kern<<<(unsigned)blocks, threads, 0, s>>>(a, d, sc, g.scratch, uin, p0);
   return cudaGetLastError();
 }
 
