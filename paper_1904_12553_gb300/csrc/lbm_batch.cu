@@ -371,10 +371,16 @@ __global__ void __launch_bounds__(BG::NTH, 1)
       }
       item = cbase + chunk - cleft--;
     }
-    else if (sched == SCHED_LISTS) item = lbeg + k < lend ? list[lbeg + k] : nitems;
+    else if (sched == SCHED_LISTS)
+      item = lbeg + k < lend ? list[rev ? lend - 1 - k : lbeg + k] : nitems;
     else item = blockIdx.x + k * gridDim.x;
     ++k;
     return item;
+  };
+  // rev: the items from the last to the first; a list from its own end, since the
+  // lists are balanced for the items that they hold
+  auto item_at = [&](int i) {
+    return items[rev && sched != SCHED_LISTS ? nitems - 1 - i : i];
   };
   const TmaItem none = {-1, 0, 0, 0, 0, 0, 0, 0};
   TmaItem d_next = none;
@@ -383,7 +389,7 @@ __global__ void __launch_bounds__(BG::NTH, 1)
     const int slot = j % S;
     const TmaItem d = d_next;
     if (d.c >= 0) {
-      d_next = i_after < nitems ? items[rev ? nitems - 1 - i_after : i_after] : none;
+      d_next = i_after < nitems ? item_at(i_after) : none;
       i_after = i_after < nitems ? next_index() : nitems;
     }
     s_slot[slot] = d;
@@ -419,7 +425,7 @@ __global__ void __launch_bounds__(BG::NTH, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     const int i0 = next_index();
     if (i0 < nitems) {
-      d_next = items[rev ? nitems - 1 - i0 : i0];
+      d_next = item_at(i0);
       i_after = next_index();
     }
     for (int j = 0; j < S; ++j) issue(j);
@@ -514,7 +520,7 @@ struct lbm_nphase_batch_t {
   int *d_list_off, *d_list, *d_counter;
   size_t items_cap, lists_cap;
   int nitems;
-  bool big;                // the state is beyond L2 (see walk_back)
+  bool big;                // states of 48 MB on: odd steps walk back (walk_back)
   lbm_nphase_batch_schedule sched;
   int max_ctas[2];         // resident CTAs per tile height (generic kernel)
   int max_ctas_tma;        // resident CTAs of the pipelined kernel
@@ -583,8 +589,8 @@ lbm_status build_schedule(lbm_nphase_batch_t *b, lbm_nphase_batch_schedule s) {
   if (s.chunk < 0) return LBM_EINVAL;
   if (s.chunk == 0) s.chunk = 1;
   if (s.ctas <= 0 || s.ctas > cap) s.ctas = cap;
-  // Cases in order of decreasing work (cost of a tile ~ N), tiles of a case
-  // consecutive (neighbouring tiles share halos in L2).
+  // Cases in order of decreasing work (cost of a tile ~ N), the tiles of a case
+  // together (neighbouring tiles share halos in L2).
   std::vector<int> order(b->n);
   std::iota(order.begin(), order.end(), 0);
   auto cost = [&](int c) {
