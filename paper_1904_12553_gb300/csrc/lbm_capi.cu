@@ -609,7 +609,7 @@ static cudaError_t step_once(lbm_nphase_t *h, cudaStream_t s, int cur) {
 constexpr int kChain[2] = {2, 32};
 
 // kChain[l] steps from buffer p (an even number: back to p) as a graph.
-static cudaError_t build_step_graph(lbm_nphase_t *h, int l, int p) {
+static cudaError_t capture_steps(lbm_nphase_t *h, int l, int p) {
   cudaError_t e = cudaSuccess;
   if (!h->cap) e = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal);
@@ -621,6 +621,17 @@ static cudaError_t build_step_graph(lbm_nphase_t *h, int l, int p) {
   if (e == cudaSuccess) e = es;
   if (e == cudaSuccess) e = cudaGraphInstantiate(&h->gexec[l][p], graph, 0);
   if (graph) cudaGraphDestroy(graph);
+  return e;
+}
+
+// The same, as a part of lbm_nphase_step that a caller does not see: in relaxed
+// mode, so that a capture under way on another stream, of this thread or of
+// another one, stays valid.
+static cudaError_t build_step_graph(lbm_nphase_t *h, int l, int p) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const cudaError_t e = capture_steps(h, l, p);
+  cudaThreadExchangeStreamCaptureMode(&mode);
   return e;
 }
 
