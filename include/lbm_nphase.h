@@ -142,8 +142,8 @@ lbm_status lbm_nphase_init(lbm_nphase_t *h, const double *c, const double *u,
  * collisions (Eqs. 24, N24) and streaming (two for FP64 grids with unequal
  * densities or Eq. N40). From nsteps >= 4 on, pairs of steps are replayed
  * from a CUDA graph captured on the handle's first such call (on a private
- * stream; call it outside any capture of your own), from nsteps >= 32 on
- * also chains of 32.
+ * stream; call it outside any capture of your own), and chains of 32 once a
+ * handle has run enough steps to repay their capture.
  * Errors: LBM_ESTATE before init or after LBM_EUNSTABLE, LBM_ECUDA. */
 lbm_status lbm_nphase_step(lbm_nphase_t *h, int64_t nsteps);
 

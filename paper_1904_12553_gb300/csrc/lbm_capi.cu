@@ -602,10 +602,12 @@ static cudaError_t step_once(lbm_nphase_t *h, cudaStream_t s, int cur) {
 
 // Steps per graph: a pair, and a chain for long runs. Back to back, graphs
 // start at multiples of about 2 us on GB300, kernels inside one graph follow
-// each other at once (0.55 us for empty ones), so a chain saves a small
-// grid's step up to 1 us: FP32 256^2 with walls 6.16 us per step in pairs,
-// 5.39 in chains of 8, 5.26 of 16, 5.27 of 32, 5.24 of 64. Chains of 32 are
-// captured when a call of at least that many steps first asks for one.
+// each other at once (0.55 us for empty ones), so a chain saves 1 to 1.6 us per
+// step (pairs / chain: FP32 64^2 N = 3 4.11 / 3.02, 512^2 N = 5 21.5 / 20.1,
+// 2048^2 268.2 / 266.7; chains of 8, 16, 64 within 2% of 32). Its capture and
+// instantiation take about 100 us, so it is built once a handle has run, or is
+// about to run, kChainPays steps from the same buffer.
+constexpr int kChainPays = 128;
 constexpr int kChain[2] = {2, 32};
 
 // kChain[l] steps from buffer p (an even number: back to p) as a graph.
@@ -635,10 +637,12 @@ static cudaError_t build_step_graph(lbm_nphase_t *h, int l, int p) {
   return e;
 }
 
-// Whether a chain from the current buffer is there, built now if need be. Not
-// while the caller captures the handle's stream: such calls replay pairs.
-static bool have_chain(lbm_nphase_t *h) {
+// Whether a chain from the current buffer is there, built now if `left` steps
+// repay it. Not while the caller captures the handle's stream: such calls
+// replay pairs.
+static bool have_chain(lbm_nphase_t *h, int64_t left) {
   if (h->gexec[1][h->cur]) return true;
+  if (h->paired[h->cur] + left < kChainPays) return false;
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (h->no_chain || cudaStreamIsCapturing(h->stream, &st) != cudaSuccess ||
       st != cudaStreamCaptureStatusNone) {
@@ -656,22 +660,27 @@ lbm_status lbm_nphase_step(lbm_nphase_t *h, int64_t nsteps) {
   if (!h->initialized || h->unstable) return LBM_ESTATE;
   int64_t t = 0;
   if (nsteps >= 4 && !h->gexec[0][0]) {
-    // one step launched directly first: the launchers' one-time setup
-    // (shared-memory attributes, occupancy) then runs outside the capture
-    cudaError_t e = step_once(h, h->stream, h->cur);
-    if (e != cudaSuccess) return cuda_fail(h, e);
-    h->cur ^= 1;
-    ++h->steps;
-    ++t;
+    // two steps launched directly first: the launchers' one-time setup
+    // (shared-memory attributes, occupancy) then runs outside the capture, and
+    // runs of even length start from the same buffer in the first call as later
+    cudaError_t e = cudaSuccess;
+    for (; t < 2; ++t) {
+      e = step_once(h, h->stream, h->cur);
+      if (e != cudaSuccess) return cuda_fail(h, e);
+      h->cur ^= 1;
+      ++h->steps;
+    }
     for (int p = 0; p < 2 && e == cudaSuccess; ++p) e = build_step_graph(h, 0, p);
     if (e != cudaSuccess) return cuda_fail(h, e);
   }
   if (h->gexec[0][0])
     for (int l = 1; l >= 0; --l)
-      for (; t + kChain[l] <= nsteps && (l == 0 || have_chain(h)); t += kChain[l]) {
+      for (; t + kChain[l] <= nsteps && (l == 0 || have_chain(h, nsteps - t));
+           t += kChain[l]) {
         cudaError_t e = cudaGraphLaunch(h->gexec[l][h->cur], h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e);
         h->steps += kChain[l];
+        if (l == 0) h->paired[h->cur] += kChain[l];
       }
   for (; t < nsteps; ++t) {
     cudaError_t e = step_once(h, h->stream, h->cur);

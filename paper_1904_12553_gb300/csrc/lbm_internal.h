@@ -177,6 +177,7 @@ struct lbm_nphase_t {
   int cuda_err;
   cudaStream_t cap;            // private stream for graph capture
   cudaGraphExec_t gexec[2][2]; // a pair, a chain of steps from buffer 0 / 1
+  int64_t paired[2];           // steps replayed in pairs from buffer 0 / 1
   bool no_chain;               // the chain's capture failed: pairs only
 };
 
