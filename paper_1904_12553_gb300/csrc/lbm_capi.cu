@@ -724,12 +724,25 @@ int state_parts(const lbm_nphase_t *h, Part out[5]) {
   return 5;
 }
 
-// Rows of nx values from pitch sp to pitch dp.
-__global__ void copy_rows_kernel(float *dst, size_t dp, const float *src, size_t sp, int nx,
-                                 size_t rows) {
-  for (size_t r = blockIdx.x * 8 + threadIdx.y; r < rows; r += (size_t)gridDim.x * 8)
-#pragma unroll 4
-    for (int x = threadIdx.x; x < nx; x += 32) dst[r * dp + x] = src[r * sp + x];
+// n dense values (rows of nx) to or from rows of pitch px, value by value in
+// dense order, eight loads of a thread in flight. n < 2^32.
+__global__ void __launch_bounds__(256) copy_rows_kernel(float *dense, float *rows, unsigned nx,
+                                                        unsigned px, unsigned n, bool pack) {
+  const size_t base = (size_t)blockIdx.x * 2048 + threadIdx.x;
+  float v[8];
+  size_t at[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const size_t i = base + k * 256;
+    const unsigned r = (unsigned)i / nx;
+    at[k] = (size_t)r * px + ((unsigned)i - r * nx);
+    if (i < n) v[k] = pack ? rows[at[k]] : dense[i];
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const size_t i = base + k * 256;
+    if (i < n) (pack ? dense[i] : rows[at[k]]) = v[k];
+  }
 }
 
 size_t part_bytes(const lbm_nphase_t *h, const Part &p) {
@@ -738,8 +751,9 @@ size_t part_bytes(const lbm_nphase_t *h, const Part &p) {
 
 // Copies a part to or from the blob's dense rows. Padded rows (FP32) are packed
 // and unpacked by a kernel, through the staging area for a blob in host memory:
-// row by row, as a 2-D copy, took up to 40 times as long (set_state from host
-// memory: 105 x 5000, N = 3 4900 -> 400 us, 1501 x 997, N = 4 2440 -> 1330).
+// as a 2-D copy, row by row, set_state took up to 40 times as long (from host
+// memory, us: 101 x 5000, N = 3 4906 -> 454, 1501 x 997, N = 4 2443 -> 1450), and
+// get_state six times on short rows (874 -> 460; long ones go as fast as dense).
 // Blobs that a kernel cannot address (another GPU's memory, addresses that are
 // no multiple of 4) take the staging area too.
 cudaError_t copy_part(const lbm_nphase_t *h, const Part &p, void *blob, bool to_blob,
@@ -749,29 +763,28 @@ cudaError_t copy_part(const lbm_nphase_t *h, const Part &p, void *blob, bool to_
     return to_blob ? cudaMemcpyAsync(blob, p.dev, part_bytes(h, p), kind, h->stream)
                    : cudaMemcpyAsync(p.dev, blob, part_bytes(h, p), kind, h->stream);
   const size_t rows = p.planes * h->g.ny * h->g.nz;
+  if (kind == cudaMemcpyDeviceToHost && nx >= 512)
+    return cudaMemcpy2DAsync(blob, nx * 4, p.dev, px * 4, nx * 4, rows, kind, h->stream);
   const size_t Vd = nx * h->g.ny * h->g.nz;
   cudaPointerAttributes at;
   bool dev = false;
   if (((uintptr_t)blob & 3u) == 0 && cudaPointerGetAttributes(&at, blob) == cudaSuccess)
     dev = at.type == cudaMemoryTypeDevice && at.device == h->device;
   cudaGetLastError();
-  const size_t fit = dev ? rows : (h->prm.N + dims(&h->prm)) * Vd * 8 / (nx * 4);
+  // rows at a time: what the staging area holds, and fewer than 2^31 values
+  size_t fit = dev ? rows : (h->prm.N + dims(&h->prm)) * Vd * 8 / (nx * 4);
+  if (fit > ((size_t)1 << 31) / px) fit = ((size_t)1 << 31) / px;
   cudaError_t e = cudaSuccess;
   for (size_t r = 0; r < rows && e == cudaSuccess; r += fit) {
-    const size_t n = rows - r < fit ? rows - r : fit;
+    const size_t n = (rows - r < fit ? rows - r : fit) * nx;
     float *state = (float *)p.dev + r * px, *user = (float *)blob + r * nx;
     float *dense = dev ? user : (float *)h->stage;
-    if (!dev && !to_blob)
-      e = cudaMemcpyAsync(dense, user, n * nx * 4, kind, h->stream);
+    if (!dev && !to_blob) e = cudaMemcpyAsync(dense, user, n * 4, kind, h->stream);
     if (e != cudaSuccess) return e;
-    const unsigned blocks = (unsigned)(n < 8 * 2432 ? (n + 7) / 8 : 2432);
-    if (to_blob)
-      copy_rows_kernel<<<blocks, dim3(32, 8), 0, h->stream>>>(dense, nx, state, px, (int)nx, n);
-    else
-      copy_rows_kernel<<<blocks, dim3(32, 8), 0, h->stream>>>(state, px, dense, nx, (int)nx, n);
+    copy_rows_kernel<<<(unsigned)((n + 2047) / 2048), 256, 0, h->stream>>>(
+        dense, state, (unsigned)nx, (unsigned)px, (unsigned)n, to_blob);
     e = cudaGetLastError();
-    if (e == cudaSuccess && !dev && to_blob)
-      e = cudaMemcpyAsync(user, dense, n * nx * 4, kind, h->stream);
+    if (e == cudaSuccess && !dev && to_blob) e = cudaMemcpyAsync(user, dense, n * 4, kind, h->stream);
   }
   return e;
 }
