@@ -256,7 +256,7 @@ def time_form(w, prec, steps, warmup, dist=None, segments=None):
         dist.barrier()
         ms = max_over_ranks(ms, dist, "cuda")
     mass, ke, _ = s.diagnostics()
-    kernel = s.step_kernel
+    kernel = s.kernels
     s.close()
     return ms, (wall0, wall1), mass, ke, kernel
 
@@ -293,15 +293,15 @@ def e2e_run(w, prec, steps):
 
 def d3q15_run(n=256, steps=100, prec="fp32"):
     """D3Q15 (three dimensions): three phases, two sphere drops R = n/6 in a
-    periodic n^3 box, z-marching 3-D kernel; FP32 storage, or 16-bit
-    storage relative to the advective and pressure parts of the
+    periodic n^3 box; FP32 storage (z-marching kernel), or 16-bit storage
+    (phi and step kernels) relative to the advective and pressure parts of the
     equilibrium."""
     import torch
     from paper_1904_12553_gb300 import Solver, workloads as W
 
     w = W.sphere_drops3(n=n, N=3, R=n / 6.0, precision=prec)
     s = Solver(w.params)
-    kernel = s.step_kernel
+    kernel = s.kernels
     s.init(w.c0)
     s.step(3)
     torch.cuda.synchronize()

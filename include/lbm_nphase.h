@@ -137,10 +137,11 @@ lbm_status lbm_nphase_init(lbm_nphase_t *h, const double *c, const double *u,
                            double p0);
 
 /* Advance nsteps >= 0 time steps (asynchronous on the handle's stream). Each
- * step is one fused kernel: zeroth moments (Eq. N28), chemical potentials
- * (Eqs. N17, N18, N31), forces, u and p (Eqs. N22_1, N23), both
- * collisions (Eqs. 24, N24) and streaming (two for FP64 grids with unequal
- * densities or Eq. N40). From nsteps >= 4 on, pairs of steps are replayed
+ * step takes zeroth moments (Eq. N28), chemical potentials (Eqs. N17, N18,
+ * N31), forces, u and p (Eqs. N22_1, N23), both collisions (Eqs. 24, N24) and
+ * streaming, in one fused kernel; in two for FP64 D2Q9 grids with unequal
+ * densities or Eq. N40, in two or, with unequal densities, three for D3Q15
+ * grids other than large FP32 boxes. From nsteps >= 4 on, pairs of steps are replayed
  * from a CUDA graph captured on the handle's first such call (on a private
  * stream; call it outside any capture of your own), and chains of 32 once a
  * handle has run enough steps to repay their capture.
@@ -202,8 +203,8 @@ typedef struct {
                           item's populations loaded while the current one is
                           computed; tile_height is then 8); needs every case
                           to satisfy the pipelined kernel's conditions
-                          (nx a multiple of 8, lbm_nphase_uses_pipelined_kernel
-                          true for it), else LBM_EINVAL */
+                          (nx a multiple of 8; lbm_nphase_uses_pipelined_kernel
+                          1 for lbm_nphase_batch_case), else LBM_EINVAL */
   int32_t chunk;       /* dynamic schedule: consecutive items taken per
                           atomic grab (0 means 1); ignored otherwise */
 } lbm_nphase_batch_schedule;
@@ -282,18 +283,22 @@ lbm_status lbm_nphase_set_state(lbm_nphase_t *h, const void *src, size_t bytes);
 /* Number of time steps taken since the last init. */
 int64_t lbm_nphase_steps_taken(const lbm_nphase_t *h);
 
-/* Which kernels lbm_nphase_step has for this handle: 1 the TMA-pipelined
- * D2Q9 kernel (FP32 and 16-bit forms, equal pure-phase densities, nx a
- * multiple of 8; FP32 grids of up to 608 tiles of 32 x 8 nodes run the
- * generic tile kernel, which is faster there), 2 the D3Q15 step split into a phi and a step kernel (equal
- * densities, every storage form), 3 the same and the z-marching D3Q15 kernel
- * with TMA-staged planes for large boxes (FP32, equal densities, N <= 4, nx a
- * multiple of 4), 0 the others (D2Q9: FP64 kernels or the generic tile
- * kernel; D3Q15, unequal densities: split into phi, C_i and step kernels).
- * Setting the environment variable LBM_NPHASE_KERNEL before
- * lbm_nphase_create to "generic" selects the generic tile kernels everywhere,
- * to "pipelined" the TMA kernels at every size of cases 1 and 3. All compute
- * the same step. */
+/* The kernels that a step of this handle launches, by name: "tile_kernel",
+ * "tile_kernel (ring warps)", "tile_kernel_tma", "step64_kernel", "pot64_kernel
+ * + coll64_kernel" (D2Q9), "phi3_kernel + step3_kernel", "phi3_kernel +
+ * pot3_kernel + step3_kernel", "march3_tma_kernel", "tile3_kernel" (D3Q15). A
+ * static string. All compute the same step. Setting the environment variable
+ * LBM_NPHASE_KERNEL before lbm_nphase_workspace_bytes and lbm_nphase_create to
+ * "generic" selects tile_kernel and tile3_kernel everywhere, to "pipelined"
+ * tile_kernel_tma and march3_tma_kernel at every size that they can run. */
+const char *lbm_nphase_step_kernels(const lbm_nphase_t *h);
+
+/* Which TMA kernel is prepared for this handle's grid, whether or not its size
+ * makes a step run it (lbm_nphase_step_kernels says what does): 1 the pipelined
+ * D2Q9 kernel (equal pure-phase densities, central scheme; 16-bit forms with nx a
+ * multiple of 8, FP32 with nx a multiple of 8 or padded rows), 3 the z-marching
+ * D3Q15 kernel with TMA-staged planes (FP32, equal densities, N <= 4, nx a
+ * multiple of 4), 2 none, D3Q15 with equal densities, 0 none. */
 int lbm_nphase_uses_pipelined_kernel(const lbm_nphase_t *h);
 
 /* Self-test of the timeout path (not part of the paper). Launches, on the

@@ -124,6 +124,8 @@ def load_library():
         lib.lbm_nphase_set_state.restype = C.c_int
         lib.lbm_nphase_uses_pipelined_kernel.argtypes = [vp]
         lib.lbm_nphase_uses_pipelined_kernel.restype = C.c_int
+        lib.lbm_nphase_step_kernels.argtypes = [vp]
+        lib.lbm_nphase_step_kernels.restype = C.c_char_p
         lib.lbm_nphase_destroy.argtypes = [vp]
         lib.lbm_nphase_strerror.argtypes = [C.c_int]
         lib.lbm_nphase_strerror.restype = C.c_char_p
@@ -270,6 +272,10 @@ def lbm_nphase_uses_pipelined_kernel(handle: int) -> int:
         C.c_void_p(handle)))
 
 
+def lbm_nphase_step_kernels(handle: int) -> str:
+    return load_library().lbm_nphase_step_kernels(C.c_void_p(handle)).decode()
+
+
 def lbm_nphase_destroy(handle: int):
     load_library().lbm_nphase_destroy(C.c_void_p(handle))
 
@@ -368,14 +374,20 @@ class Solver:
         lbm_nphase_set_state(self.handle, blob.data_ptr(), blob.numel())
 
     @property
+    def kernels(self) -> str:
+        """The kernels that a step launches, by name."""
+        return lbm_nphase_step_kernels(self.handle)
+
+    @property
     def pipelined(self) -> bool:
-        """True if steps run the TMA-pipelined D2Q9 kernel."""
+        """True if the TMA-pipelined D2Q9 kernel is prepared for this grid;
+        small FP32 grids run the generic one all the same (see kernels)."""
         return lbm_nphase_uses_pipelined_kernel(self.handle) == 1
 
     @property
     def step_kernel(self) -> str:
-        """Name of the step's kernels (2 and 3: the D3Q15 kernels, split or,
-        for large FP32 boxes, z-marching)."""
+        """Name of the family that lbm_nphase_uses_pipelined_kernel reports as
+        prepared; what a step launches is in kernels."""
         return {1: "pipelined (TMA)", 2: "z-marching 3-D",
                 3: "z-marching 3-D (TMA)"}.get(
             lbm_nphase_uses_pipelined_kernel(self.handle), "generic tile")

@@ -944,7 +944,23 @@ lbm_status lbm_nphase_diagnostics(lbm_nphase_t *h, double *mass, double *ke,
 
 int lbm_nphase_uses_pipelined_kernel(const lbm_nphase_t *h) {
   if (!h) return 0;
-  return h->g.use_tma && h->g.nx % 8 == 0 ? 1 : (h->g.tma3 ? 3 : (h->g.march3 ? 2 : 0));
+  return h->g.use_tma ? 1 : (h->g.tma3 ? 3 : (h->g.march3 ? 2 : 0));
+}
+
+const char *lbm_nphase_step_kernels(const lbm_nphase_t *h) {
+  if (!h) return "";
+  switch (lbm::step_path(h->prec, h->prm.N, h->g, h->nonunif)) {
+    case lbm::STEP_TILE: return "tile_kernel";
+    case lbm::STEP_TILE_RING: return "tile_kernel (ring warps)";
+    case lbm::STEP_TMA: return "tile_kernel_tma";
+    case lbm::STEP_FP64: return "step64_kernel";
+    case lbm::STEP_FP64_SPLIT: return "pot64_kernel + coll64_kernel";
+    case lbm::STEP_TILE3: return "tile3_kernel";
+    case lbm::STEP_SPLIT3: return "phi3_kernel + step3_kernel";
+    case lbm::STEP_SPLIT3_NU: return "phi3_kernel + pot3_kernel + step3_kernel";
+    case lbm::STEP_MARCH3: return "march3_tma_kernel";
+  }
+  return "";
 }
 
 int64_t lbm_nphase_steps_taken(const lbm_nphase_t *h) { return h ? h->steps : 0; }

@@ -85,12 +85,6 @@ __device__ __forceinline__ void stencil3(const T *s, int lz, int ly, int lx,
   lap = T(6) * l;
 }
 
-template <int P>
-__device__ __forceinline__ typename Prec<P>::T load_hm3(const KArgs<P> &a, int i,
-                                                        int k, size_t q) {
-  return to_T(ldg(a.hm_in + ((size_t)(i * 14 + k - 1)) * a.V + q));
-}
-
 // 16-bit forms store every moving population relative to the advective (and
 // for g the pressure) part of its equilibrium at the node it was streamed
 // from, as in two dimensions (cdotu, adv_units, g_refp there): c_k . u with
@@ -1358,18 +1352,6 @@ __global__ void init3_pop_kernel(const KArgs3<P> A, const KArgs<LBM_FP64> d,
   }
 }
 
-// Whether the TMA-staged z-marching kernel beats the split step: it reads h
-// once, but needs columns enough to fill the GPU and few idle lanes in them.
-// us per step, march / split, N = 3: 64^3 29.8 / 23.8, 96^3 86.5 / 87.2, 128^3
-// 184 / 199, 160^3 329 / 384, 256^3 1290 / 1538, 40 x 200 x 120 (62% of the
-// columns' lanes) 152 / 114; N = 2: 128^3 133 / 124, 192 x 192 x 200 401 / 424.
-inline bool march3_pays(const Grid &g, int NP) {
-  if (!g.tma3) return false;
-  if (g.tma_all) return true;
-  const long long cols = (long long)tiles_x(g.nx) * 32 * ((g.ny + MY3 - 1) / MY3) * MY3;
-  return g.V >= ((size_t)1 << (NP >= 2 ? 20 : 22)) && (long long)g.nx * g.ny * 5 >= cols * 4;
-}
-
 template <int P, int NP, bool NU, bool WALL>
 cudaError_t launch_tile3_t(const Consts &c, const Grid &g, int cur, int mode,
                            const Outputs &o, cudaStream_t s) {
@@ -1388,9 +1370,10 @@ cudaError_t launch_tile3_t(const Consts &c, const Grid &g, int cur, int mode,
     macro3_kernel<P, NP, NU, WALL><<<tiles, tblock, 0, s>>>(A);
     return cudaGetLastError();
   }
-  if (mode == MODE_STEP && g.split3) {
+  const StepPath path = step_path(P, c.N, g, NU);
+  if (mode == MODE_STEP && path != STEP_TILE3) {
     if constexpr (P == LBM_FP32 && NP <= 3 && !NU) {
-      if (march3_pays(g, NP)) {
+      if (path == STEP_MARCH3) {
         // slabs of z planes: enough CTAs to fill the GPU (~1216), at least 8
         // planes per slab (each slab sums phi on two extra planes)
         const int txy = tiles_x(g.nx) * ((g.ny + MY3 - 1) / MY3);

@@ -74,7 +74,7 @@ struct Grid {
   double *scratch;  // FP64 staging of host inputs and outputs ([N + D][V]);
                     // initialisation keeps phi_i there ([N-1][V])
   int grad_scheme;  // 0: central (Eq. N31a), 1: mixed (Eq. N40)
-  bool use_tma;     // pipelined kernel usable for this grid
+  bool use_tma;     // pipelined kernel prepared (tma[] encoded): see step_path
   bool step64;      // D2Q9 step by the FP64 kernels (lbm_step64.cuh)
   bool split3;      // D3Q15 step by the split or z-marching kernels
   bool march3;      // ... with equal densities
@@ -151,6 +151,49 @@ inline bool tma_pays(int N, int nx, int ny) {
 // (73 x 40000 173 / 203). 2 x 1 and 4 x 1 are slower than both at 2048^2.
 inline bool tma_three_stages(int nx, int ny) {
   return tiles_of(nx, ny) > 33 * 152 && (nx >= 96 || nx % 8 != 0);
+}
+// FP32 grids whose tiles are all resident at once, ring_ctas per SM, take the
+// generic kernel with halo-ring warps (see there).
+constexpr int ring_ctas(int NP, bool NU, bool G40) {
+  return NP <= (NU && G40 ? 0 : NU || G40 ? 2 : 3) ? 2 : 1;
+}
+// Whether the TMA-staged z-marching kernel beats the split step: it reads h
+// once, but needs columns enough to fill the GPU and few idle lanes in them.
+// us per step, march / split, N = 3: 64^3 29.8 / 23.8, 96^3 86.5 / 87.2, 128^3
+// 184 / 199, 160^3 329 / 384, 256^3 1290 / 1538, 40 x 200 x 120 (62% of the
+// columns' lanes) 152 / 114; N = 2: 128^3 133 / 124, 192 x 192 x 200 401 / 424.
+inline bool march3_pays(const Grid &g, int NP) {
+  if (!g.tma3) return false;
+  if (g.tma_all) return true;
+  const long long cols = (long long)tiles_x(g.nx) * 32 * ((g.ny + 7) / 8) * 8;
+  return g.V >= ((size_t)1 << (NP >= 2 ? 20 : 22)) && (long long)g.nx * g.ny * 5 >= cols * 4;
+}
+// The kernels of one step: what the launchers run and lbm_nphase_step_kernels
+// reports.
+enum StepPath {
+  STEP_TILE,        // tile_kernel
+  STEP_TILE_RING,   // ... with halo-ring warps
+  STEP_TMA,         // tile_kernel_tma
+  STEP_FP64,        // step64_kernel
+  STEP_FP64_SPLIT,  // pot64_kernel, coll64_kernel
+  STEP_TILE3,       // tile3_kernel
+  STEP_SPLIT3,      // phi3_kernel, step3_kernel
+  STEP_SPLIT3_NU,   // phi3_kernel, pot3_kernel, step3_kernel
+  STEP_MARCH3       // march3_tma_kernel
+};
+inline StepPath step_path(int prec, int N, const Grid &g, bool nonunif) {
+  const bool g40 = g.grad_scheme == 1;
+  if (g.lattice == 1) {
+    if (!g.split3) return STEP_TILE3;
+    if (march3_pays(g, N - 1)) return STEP_MARCH3;
+    return nonunif ? STEP_SPLIT3_NU : STEP_SPLIT3;
+  }
+  if (g.step64) return nonunif || g40 ? STEP_FP64_SPLIT : STEP_FP64;
+  if (g.use_tma && (prec != LBM_FP32 || g.tma_all || tma_pays(N, g.nx, g.ny))) return STEP_TMA;
+  if (prec == LBM_FP32 && g.ring_warps &&
+      tiles_of(g.nx, g.ny) <= 152 * ring_ctas(N - 1, nonunif, g40))
+    return STEP_TILE_RING;
+  return STEP_TILE;
 }
 // CTAs of the generic step / moments / diagnostics kernel of a grid
 inline size_t tiles_total(int lattice, int nx, int ny, int nz) {

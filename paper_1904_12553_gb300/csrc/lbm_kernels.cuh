@@ -813,7 +813,9 @@ __device__ __forceinline__ void phi_global(const KArgs<P> &a, int sx, int sy,
 // time step; MODE_MOMENTS: write the macroscopic fields; MODE_DIAG: per-CTA
 // partial sums of the diagnostics).
 // ---------------------------------------------------------------------------
-// Resident CTAs the FP32 kernel is compiled for, and whether a node's NS
+// Resident CTAs the kernel is compiled for (16-bit: what they were without a
+// bound; a register more than it allows cost BF16 705 x 503, N = 5, walls 40 ->
+// 55 us per step), and, FP32, whether a node's NS
 // populations and u(t-1) are loaded before the halo ring (one memory latency
 // instead of two: what counts on a grid of one wave of tiles) where registers
 // are left for them. us per step in 2 / 3 / 4 CTAs (e: loaded early): N = 3,
@@ -843,9 +845,6 @@ template <int P, int NP, bool NU, bool G40> struct TileMin {
 // 150^2 4.13 / 4.99, N = 5, 200 x 150 5.71 / 6.55.
 // Beyond one wave the occupancy it gives up costs more: unequal N = 2, 400 x
 // 200 (325 tiles), 7.96 with 4 warps in 3 CTAs / 6.99.
-constexpr int ring_ctas(int NP, bool NU, bool G40) {
-  return NP <= (NU && G40 ? 0 : NU || G40 ? 2 : 3) ? 2 : 1;
-}
 constexpr int ring_rw(bool NU, bool G40) {  // ring of radius 1, 2 or 3: 84, 176 or 276 positions
   return NU && G40 ? 9 : NU || G40 ? 6 : 3;
 }
@@ -1797,12 +1796,13 @@ cudaError_t launch_tma_t(const KArgs<P> &a, const Grid &g, int cur, cudaStream_t
 template <int P, int NP, bool NU, bool WALL>
 cudaError_t launch_tile_t(const Consts &c, const Grid &g, int cur, int mode,
                           const Outputs &o, cudaStream_t s) {
+  const StepPath path = mode == MODE_STEP ? step_path(P, c.N, g, NU) : STEP_TILE;
   if constexpr (P == LBM_FP64)
-    if (mode == MODE_STEP && g.step64) return launch_step64<NP, NU, WALL>(c, g, cur, s);
+    if (path == STEP_FP64 || path == STEP_FP64_SPLIT)
+      return launch_step64<NP, NU, WALL>(c, g, cur, s);
   const KArgs<P> a = make_args<P>(c, g, cur, mode, o);
   if constexpr (P != LBM_FP64 && !NU) {
-    if (mode == MODE_STEP && g.use_tma &&
-        (P != LBM_FP32 || g.tma_all || tma_pays(c.N, g.nx, g.ny))) {
+    if (path == STEP_TMA) {
       if constexpr (P == LBM_FP32 && NP == 2)
         if (tma_three_stages(g.nx, g.ny)) return launch_tma_t<P, NP, WALL, 3>(a, g, cur, s);
       return launch_tma_t<P, NP, WALL, TmaGeom<P>::S>(a, g, cur, s);
@@ -1810,11 +1810,9 @@ cudaError_t launch_tile_t(const Consts &c, const Grid &g, int cur, int mode,
   }
   dim3 grid(tiles_x(g.nx), tiles_y(g.ny)), block(BX, BY);
   if constexpr (P == LBM_FP32) {
-    const bool g40 = g.grad_scheme == 1;
-    if (mode == MODE_STEP && g.ring_warps &&
-        (long long)tiles_x(g.nx) * tiles_y(g.ny) <= 152 * ring_ctas(NP, NU, g40)) {
+    if (path == STEP_TILE_RING) {
       constexpr int RW = ring_rw(NU, false), RW40 = ring_rw(NU, true);
-      if (g40)
+      if (g.grad_scheme == 1)
         tile_kernel<P, NP, NU, WALL, true, RW40><<<grid, dim3(BX, BY + RW40), 0, s>>>(a);
       else
         tile_kernel<P, NP, NU, WALL, false, RW><<<grid, dim3(BX, BY + RW), 0, s>>>(a);
