@@ -48,13 +48,14 @@ def alg_bytes_per_node(N: int, prec: str) -> int:
 
 # FP64 instructions one node-step executes in the FP64 form at N=5 (ncu: 11.80 M
 # warp instructions of the step kernel on the 1024x1024 droplets and interfaces
-# case, all of them DFMA; profiles/step64_kernel_fp64_n5_1024.md). Sums and
-# products are executed as fused multiply-adds, so a slot is counted as two
-# operations whatever it computes.
-FP64_FLOP_PER_NODE_N5 = 2 * 360.0
-# FP64 ALU peak derived from the GB300's unit counts and clock: 152 SMs x
-# 2 FP64 FMA lanes per SM per clock x 2 FLOP x 2070 MHz = 1.2586 TFLOP/s.
-FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
+# case, all of them DFMA; profiles/step64_kernel_fp64_n5_1024.md). They do the
+# work of 679.5 additions and multiplications in a kernel without folded
+# constants; sums and products are issued as fused multiply-adds, so what is
+# reported is instruction slots, not operations.
+FP64_INSTR_PER_NODE_N5 = 360.0
+# FP64 issue peak derived from the GB300's unit counts and clock: 152 SMs x
+# 2 lanes per SM per clock x 2070 MHz = 629.3 G instructions/s.
+FP64_PEAK_GINSTR = 152 * 2 * 2.070
 
 
 def peaks():
@@ -493,13 +494,12 @@ def run_ours(args, dist, rank, world):
                 "alg_bytes_per_node": fB, "kernel": fkernel,
                 "hbm_frac": fB * V / (fstep / 1e3) / 1e9 / peak}
             if prec == "fp64" and N == 5:
-                tf = FP64_FLOP_PER_NODE_N5 * V / (fstep / 1e3) / 1e12
+                gi = FP64_INSTR_PER_NODE_N5 * V / (fstep / 1e3) / 1e9
                 forms[prec]["roofline"] = {
-                    "bound": "alu", "achieved": tf, "unit": "TFLOP/s",
-                    "peak": FP64_PEAK_TFLOPS, "frac": tf / FP64_PEAK_TFLOPS,
-                    "flop_per_node": FP64_FLOP_PER_NODE_N5,
-                    "peak_kind": "derived (152 SMs x 2 FP64 FMA/clk x "
-                                 "2070 MHz)"}
+                    "bound": "alu", "achieved": gi, "unit": "G FP64 instructions/s",
+                    "peak": FP64_PEAK_GINSTR, "frac": gi / FP64_PEAK_GINSTR,
+                    "instructions_per_node": FP64_INSTR_PER_NODE_N5,
+                    "peak_kind": "derived (152 SMs x 2 FP64 lanes x 2070 MHz)"}
     if not args.quick:
         forms["batch"] = batch_run()
         for prec3 in ("fp32", "bf16", "fp16"):

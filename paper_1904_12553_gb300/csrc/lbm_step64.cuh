@@ -30,7 +30,10 @@
 // equal densities 1064 -> 615 (494 -> 360 FP64 instructions per node; 592 is
 // the FP64 units' time for them); N = 3, 128^2 26.6 -> 11.3; N = 3, 150^2
 // unequal densities with walls 35.9 -> 20.5; N = 5, 200 x 320 unequal
-// densities, Eq. N40 156 -> 69.
+// densities, Eq. N40 156 -> 69. Largest error against a run in 80 bits (128^2, 150^2
+// unequal densities, 200 x 320 Eq. N40, three starts each): u 11.8e-15 -> 8.9e-15
+// of its largest value, p 12.8e-15 -> 9.6e-15, phi the same; both kernels differ
+// from a 64-bit model by as much as that model from the 80-bit run.
 #pragma once
 
 namespace lbm {
