@@ -895,9 +895,12 @@ __global__ void __launch_bounds__(NT + 32 * RW,
           node_phi<P>(hreg[i][0], &hreg[i][1], pp, perr[i], a.sh_ld);
     }
   }
+  // the node's offset; the 16-bit forms, short of registers, form it again where
+  // it is used
+  auto own = [&] { return (size_t)(active ? gy : 0) * a.px + (active ? gx : 0); };
+  size_t q = own();
   T g[9], up[2];
   auto load_rest = [&] {  // the node's NS populations and u(t-1)
-    const size_t q = (size_t)(active ? gy : 0) * a.px + (active ? gx : 0);
     if (active) {
       load_g_node<P, WALL>(a, gx, gy, q, g);
     } else {
@@ -957,7 +960,7 @@ __global__ void __launch_bounds__(NT + 32 * RW,
 
   if (ring_warp) return;
   // 4. Own node: stencils, C_i, forces, u, p.
-  const size_t q = (size_t)(active ? gy : 0) * a.px + (active ? gx : 0);
+  if (Prec<P>::MIX) q = own();
   if (!EARLY) load_rest();
   NodeMac<P, NP> m;
   node_macros<P, NP, NU, SW, CW, G40>(a, &sphi[0][0], SH * SW, &sC[0][0],
