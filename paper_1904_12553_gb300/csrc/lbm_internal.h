@@ -136,11 +136,13 @@ inline long long tiles_of(int nx, int ny) { return (long long)tiles_x(nx) * tile
 // and 2048^2 109 / 135, 161 / 211, 221 / 260, 265 / 360 at N = 2..5. Tiles
 // with idle lanes fill a whole stage all the same: grids up to 63 wide (57 x
 // 40000, N = 5 267 / 244; 8 x 40000, N = 3 78 / 37) or with fewer than 60% of
-// the lanes in use (20001 x 9, N = 4 18.0 / 14.4; N = 4 also 65 x 5000, 68%,
-// 29.7 / 26.5) stay on the generic kernel.
+// the lanes in use stay on the generic kernel; N = 4, whose pipelined step gains
+// least, counts live lanes only (20001 x 12, 75% 19.8 / 15.2; 65 x 5000, 68% 29.7 /
+// 26.5).
 inline bool tma_pays(int N, int nx, int ny) {
-  const long long t = tiles_of(nx, ny), line = N == 2 ? 1216 : N == 4 ? 1140 : 912;
-  return nx >= 64 && t > line && (long long)nx * ny * 100 >= t * 256 * (N == 4 ? 70 : 60);
+  const long long t = tiles_of(nx, ny), nodes = (long long)nx * ny;
+  if (N == 4) return nx >= 64 && nodes > 1140 * 256 && nodes * 100 >= t * 256 * 70;
+  return nx >= 64 && t > (N == 2 ? 1216 : 912) && nodes * 100 >= t * 256 * 60;
 }
 // N = 3: three stages of 49 KB and one CTA per SM where the state is far beyond
 // L2, else two and two CTAs (216 KB, which leave L1 little for the stores, but

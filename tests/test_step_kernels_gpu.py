@@ -92,7 +92,8 @@ CASES += [(N, sh, "fp32", 0, 0, None, k) for N, sh, k in [
     (3, (768, 304), "tile_kernel"), (3, (773, 306), "tile_kernel_tma"),
     (4, (960, 304), "tile_kernel"), (4, (955, 312), "tile_kernel_tma"),
     (5, (768, 304), "tile_kernel"), (5, (771, 309), "tile_kernel_tma"),
-    (4, (65, 5001), "tile_kernel"), (3, (20001, 9), "tile_kernel")]]
+    (4, (65, 5001), "tile_kernel"), (4, (20001, 12), "tile_kernel"), (3, (20001, 9), "tile_kernel"),
+    (4, (20001, 17), "tile_kernel_tma")]]
 
 
 @pytest.mark.parametrize("N,shape,prec,nu,g40,env,want", CASES)
