@@ -114,7 +114,9 @@ lbm_status lbm_nphase_derive(const lbm_nphase_params *params,
                              lbm_nphase_model *out);
 
 /* Bytes of device workspace a handle with these parameters needs (0 if the
- * parameters are invalid). */
+ * parameters are invalid). FP32 D2Q9 grids on the pipelined kernel have their
+ * rows padded to 8 nodes; a workspace that is too small for that, but holds dense
+ * rows, is accepted too, and the grid then runs on the generic kernel. */
 size_t lbm_nphase_workspace_bytes(const lbm_nphase_params *params);
 
 /* Create a handle on the current CUDA device. `d_workspace` is caller-owned
